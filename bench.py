@@ -39,7 +39,7 @@ from workloads import generators as gen  # noqa: E402
 METRIC = "merged_vertices_per_s"
 UNIT = "vertices/s"
 SEARCH_SRC = [os.path.join(ROOT, "paper_2602_17099_gb300", "csrc", f)
-              for f in ("search_impl.cuh", "search.cu", "search_jobs.cu")]
+              for f in ("search_impl.cuh", "search.cu", "codes.cu")]
 PROFILE = os.path.join(ROOT, "profiles", "search_kernel_sift2x500k.txt")
 PRUNE_SRC = [os.path.join(ROOT, "paper_2602_17099_gb300", "csrc", f)
              for f in ("prune.cu", "common.cuh")]

@@ -8,7 +8,9 @@
  *   device; "host" pointers are ordinary CPU memory.  The caller owns every
  *   buffer it passes in.  Scratch memory is taken from a per-device workspace
  *   that the library grows on demand and keeps until rnsm_release_workspace()
- *   or process exit.
+ *   or process exit.  Calls that search dimensions of 64 and more also keep a
+ *   byte per component of their rows (coded rows, kept and released alike; if
+ *   there is no memory for them the searches read the FP32 rows alone).
  * - Vectors are row-major float32, rows contiguous, 16-byte aligned (dim must
  *   be a multiple of 4, at most 1024).  Calls that search (rnsm_search,
  *   rnsm_expand, rnsm_build_segment, rnsm_merge) need a dimension the search
@@ -34,6 +36,8 @@
  *   keep the fastest for the process; every variant gives the same results.
  *   Environment variables read at each call (none changes a result):
  *     RNSM_SEARCH_VARIANT=v   force search launch variant v (0..3)
+ *     RNSM_SEARCH_CODES=c     coded rows in the searches: 0 none, 1 only as a
+ *                             filter, 2 (default) alone where they are exact
  *     RNSM_PRUNE_VARIANT=v    force prune variant v where it applies (0 the
  *                             FP32 triangle, 1 the pair tile, 2 the general
  *                             tile, 3 the FP32 walk)
@@ -73,7 +77,8 @@ typedef enum {
 typedef enum { RNSM_METRIC_L2 = 0, RNSM_METRIC_IP = 1 } rnsm_metric;
 
 /* Arithmetic of the candidate-by-candidate prune tiles (Section 4.2,
- * UpdateGraph).  Searches always run in FP32.  BF16 and FP8 tiles run on the
+ * UpdateGraph).  Searches always decide in FP32 (a byte code of the rows only
+ * settles, with a bound, which distances cannot matter).  BF16 and FP8 tiles run on the
  * tensor cores and every decision a tile cannot settle within its error bound
  * is re-decided with the FP32 distance, so the result equals the FP32 one. */
 typedef enum { RNSM_PREC_FP32 = 0, RNSM_PREC_BF16 = 1, RNSM_PREC_FP8 = 2 } rnsm_precision;
@@ -224,7 +229,8 @@ RNSM_API rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_
                        const mos_edge *plan, int32_t n_plan, int32_t *out_adj, void *stream,
                        rnsm_stats *stats);
 
-/* Bytes of device workspace rnsm_merge takes for these inputs. */
+/* Bytes of device workspace rnsm_merge takes for these inputs (without the
+ * coded rows: a byte per component more). */
 RNSM_API size_t rnsm_workspace_size(const rnsm_segment *segs, int32_t m, const rnsm_params *p);
 
 /* Frees the calling device's workspace (after synchronising). */

@@ -126,6 +126,8 @@ struct Ctl {
     unsigned long long *tile_tests;  // occlusion tests evaluated by the tensor-core tiles
     unsigned int *tile_err;  // [4] tile error statistics (see rnsm_stats)
     int32_t *scratch_i;      // misc int
+    CodeStats *code_stats;   // coded rows of the call
+    CodeParams *code_params;
     int32_t *kernel_ran = nullptr;  // host [2]: prune variant of the last S6 / S7 call
 };
 
@@ -192,6 +194,8 @@ void take_ctl(Bump &b, Ctl &c, int64_t max_owners = 0) {
     c.tile_tests = b.take<unsigned long long>(1);
     c.tile_err = b.take<unsigned int>(4);
     c.scratch_i = b.take<int32_t>(4);
+    c.code_stats = b.take<CodeStats>(1);
+    c.code_params = b.take<CodeParams>(1);
 }
 
 rnsm_status ctl_reset(const Ctl &c, cudaStream_t st) {
@@ -277,6 +281,87 @@ rnsm_status validate_on_device(const float *v, int64_t n, int32_t dim, const int
     CK(launch_validate_vecs(v, n * dim, c.err, st));
     if (adj && r_in > 0) CK(launch_validate_graph(adj, n, r_in, c.err, st));
     return RNSM_OK;
+}
+
+// ------------------------------------------------------------- coded rows
+//
+// A byte per dimension of every row of the call, in a grow-only buffer of its
+// own: unlike the workspace it may be missing (no memory: FP32 searches).
+
+DevWs g_codes[kMaxDev];
+
+struct Codes {
+    uint8_t *rows = nullptr;   // coded rows by global id
+    int32_t mode = kCodeNone;
+};
+
+// RNSM_SEARCH_CODES: 0 FP32 rows only, 1 never by codes alone.
+int codes_allowed() {
+    const char *f = getenv("RNSM_SEARCH_CODES");
+    return f && f[0] >= '0' && f[0] <= '2' ? f[0] - '0' : 2;
+}
+
+uint8_t *codes_acquire(size_t bytes, cudaStream_t st) {
+    DevWs &w = g_codes[cur_device()];
+    if (w.size < bytes) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return nullptr;
+        if (w.ptr) {
+            cudaDeviceSynchronize();
+            cudaFree(w.ptr);
+        }
+        w.ptr = nullptr;
+        w.size = 0;
+        if (cudaMalloc(&w.ptr, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            w.ptr = nullptr;
+            return nullptr;
+        }
+        w.size = bytes;
+    }
+    return static_cast<uint8_t *>(w.ptr);
+}
+
+// Validates the rows of the table's first `checked` segments (the error word is
+// read by the caller's check) and, where it pays, codes all of them; *params is
+// valid after that check.  evals: distances that the call's searches are
+// expected to compute.  A row's code costs what some 8 evaluations gain (a pass
+// over 5 bytes a dimension against 3 gathered bytes and most of the arithmetic).
+rnsm_status code_table(const SegTable &t, int32_t dim, int32_t metric, int32_t checked, int64_t evals,
+                       const Ctl &c, cudaStream_t st, Codes &cd, CodeParams *params) {
+    const int64_t n = t.off[t.m];
+    cd = Codes();
+    if (codes_dim_ok(dim) && codes_allowed() > 0 && evals >= 8 * n && n < INT32_MAX)
+        cd.rows = codes_acquire((size_t)n * dim, st);
+    if (!cd.rows) {
+        for (int32_t s = 0; s < checked; ++s)
+            CK(launch_validate_vecs(t.base[s], (t.off[s + 1] - t.off[s]) * dim, c.err, st));
+        return RNSM_OK;
+    }
+    CK(launch_code_scan(t, dim, checked, c.code_stats, c.err, st));
+    CK(launch_code_rows(t, dim, metric, cd.rows, c.code_stats, c.code_params, st));
+    CK(cudaMemcpyAsync(params, c.code_params, sizeof(CodeParams), cudaMemcpyDeviceToHost, st));
+    return RNSM_OK;
+}
+
+// After the check: how the searches use the codes.
+void code_mode(Codes &cd, const CodeParams &p, int32_t dim, int32_t metric) {
+    cd.mode = kCodeNone;
+    if (!cd.rows) return;
+    if (p.exact && metric == RNSM_METRIC_L2 && dim <= 256 && codes_allowed() > 1) cd.mode = kCodeExact;
+    else if (p.useful) cd.mode = kCodeFilter;
+}
+
+// A beam search evaluates some 16 vertices per entry of its beam.
+int64_t search_evals(int64_t queries, int32_t ef) { return 16 * queries * ef; }
+
+SegTable one_table(const float *vecs, int64_t n) {
+    SegTable tab;
+    std::memset(&tab, 0, sizeof(tab));
+    tab.base[0] = vecs;
+    tab.off[1] = n;
+    tab.m = 1;
+    return tab;
 }
 
 SearchArgs search_defaults() {
@@ -404,6 +489,9 @@ void rnsm_release_workspace(void) {
     }
     g_ws[dev].ptr = nullptr;
     g_ws[dev].size = 0;
+    if (g_codes[dev].ptr) cudaFree(g_codes[dev].ptr);
+    g_codes[dev].ptr = nullptr;
+    g_codes[dev].size = 0;
 }
 
 rnsm_status mos_plan(int32_t m, const int64_t *sizes, const float *centroids, int32_t D,
@@ -496,10 +584,23 @@ rnsm_status rnsm_search(const float *vecs, int64_t n, int32_t dim, const int32_t
     TRY(ws_acquire(b.off, b));
     take_ctl(b, c);
     TRY(ctl_reset(c, st));
-    TRY(validate_on_device(vecs, n, dim, adj, r_in, c, st));
+    // the queries are coded with the rows (on one grid), but not checked
+    SegTable tab = one_table(vecs, n);
+    tab.base[1] = queries;
+    tab.off[2] = n + nq;
+    tab.m = 2;
+    Codes codes;
+    CodeParams code_params;
+    TRY(code_table(tab, dim, metric, 1, nq > kLatencyQueries ? search_evals(nq, ef) : 0, c, st, codes, &code_params));
+    if (adj && r_in > 0) CK(launch_validate_graph(adj, n, r_in, c.err, st));
     CK(launch_validate_ids(seeds, nq * n_seeds, n, 1, c.err, st));  // -1 or a vertex
     TRY(check_err_word(c, st));
+    code_mode(codes, code_params, dim, metric);
     SearchArgs a = search_defaults();
+    a.code_mode = codes.mode;
+    a.code_params = c.code_params;
+    a.codes = codes.rows;
+    a.qcodes = codes.rows + (codes.rows ? (size_t)n * dim : 0);
     a.base = vecs;
     a.n_base = n;
     a.adj = adj;
@@ -539,9 +640,16 @@ rnsm_status rnsm_expand(const float *vecs, int64_t n, int32_t dim, const int32_t
     TRY(ws_acquire(b.off, b));
     take_ctl(b, c);
     TRY(ctl_reset(c, st));
-    TRY(validate_on_device(vecs, n, dim, adj, r_in, c, st));
+    Codes codes;
+    CodeParams code_params;
+    TRY(code_table(one_table(vecs, n), dim, metric, 1, search_evals(n, k_plus + 1), c, st, codes, &code_params));
+    if (adj && r_in > 0) CK(launch_validate_graph(adj, n, r_in, c.err, st));
     TRY(check_err_word(c, st));
+    code_mode(codes, code_params, dim, metric);
     SearchArgs a = search_defaults();
+    a.code_mode = codes.mode;
+    a.code_params = c.code_params;
+    a.codes = a.qcodes = codes.rows;
     a.base = vecs;
     a.n_base = n;
     a.adj = adj;
@@ -743,8 +851,12 @@ rnsm_status rnsm_build_segment(const float *vecs, int64_t n, int32_t dim, const 
     int32_t *order, *cand, *eu, *ev;
     std::tie(order, cand, eu, ev) = carve(b);
     TRY(ctl_reset(c, st));
-    TRY(validate_on_device(vecs, n, dim, nullptr, 0, c, st));
+    const SegTable tab = one_table(vecs, n);
+    Codes codes;
+    CodeParams code_params;
+    TRY(code_table(tab, dim, p.metric, 1, search_evals(n, p.L), c, st, codes, &code_params));
     TRY(check_err_word(c, st));
+    code_mode(codes, code_params, dim, p.metric);
     {
         std::vector<int32_t> h((size_t)n);
         int64_t k = 0;
@@ -755,11 +867,6 @@ rnsm_status rnsm_build_segment(const float *vecs, int64_t n, int32_t dim, const 
         CK(launch_fill(out_adj, n * p.R, -1, st));
         CK(cudaStreamSynchronize(st));
     }
-    SegTable tab;
-    std::memset(&tab, 0, sizeof(tab));
-    tab.base[0] = vecs;
-    tab.off[1] = n;
-    tab.m = 1;
     int64_t inserted = 1;
     while (inserted < n) {
         int64_t bsz = inserted < B ? inserted : B;
@@ -776,6 +883,9 @@ rnsm_status rnsm_build_segment(const float *vecs, int64_t n, int32_t dim, const 
         a.nq = bsz;
         a.seed_mode = kSeedConst;
         a.seed_const = entry;
+        a.code_mode = codes.mode;
+        a.code_params = c.code_params;
+        a.codes = a.qcodes = codes.rows;
         a.ef = p.L;
         a.k = p.L;
         a.out_ids = cand;
@@ -1051,10 +1161,12 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
     std::memset(&tab, 0, sizeof(tab));
     tab.m = m;
     int64_t off = 0, nmax = 0;
+    int32_t r_in_max = 0;   // sizes the searches' visited tables
     for (int32_t s = 0; s < m; ++s) {
         tab.base[s] = segs[s].vecs;
         tab.off[s] = off;
         off += segs[s].n;
+        r_in_max = std::max(r_in_max, segs[s].r_in);
         nmax = segs[s].n > nmax ? segs[s].n : nmax;
     }
     tab.off[m] = off;
@@ -1080,9 +1192,35 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
     int32_t kernel_ran[2] = {-1, -1};
     c.kernel_ran = kernel_ran;
     TRY(ctl_reset(c, st));
+    const bool cm = (p.flags & RNSM_FLAG_CM) != 0;
+    std::vector<int32_t> srcs;            // source segments in order of first use
+    std::vector<char> is_src((size_t)m, 0);
+    for (const PlanEdge &e : pl)
+        if (!is_src[(size_t)e.src]) {
+            is_src[(size_t)e.src] = 1;
+            srcs.push_back(e.src);
+        }
+    Codes codes;
+    CodeParams code_params;
+    int64_t evals = 0;
+    for (const PlanEdge &e : pl) evals += search_evals(segs[e.src].n, cm ? p.L : p.ef_slide);
+    if (!cm)
+        for (int32_t s : srcs) evals += search_evals(segs[s].n, p.k_plus + 1);
+    TRY(code_table(tab, dim, p.metric, m, evals, c, st, codes, &code_params));
     for (int32_t s = 0; s < m; ++s)
-        TRY(validate_on_device(segs[s].vecs, segs[s].n, dim, segs[s].adj, segs[s].r_in, c, st));
+        if (segs[s].adj && segs[s].r_in > 0)
+            CK(launch_validate_graph(segs[s].adj, segs[s].n, segs[s].r_in, c.err, st));
     TRY(check_err_word(c, st));
+    code_mode(codes, code_params, dim, p.metric);
+    auto use_codes = [&](SearchArgs &a) {
+        a.code_mode = codes.mode;
+        a.code_params = c.code_params;
+    };
+    auto code_job = [&](SearchJob &j, int32_t src, int32_t dst) {
+        if (codes.mode == kCodeNone) return;
+        j.codes = codes.rows + tab.off[dst] * dim;
+        j.qcodes = codes.rows + tab.off[src] * dim;
+    };
     for (int32_t s = 0; s < m; ++s)
         CK(launch_init_lists(segs[s].adj, segs[s].n, segs[s].r_in, (int32_t)tab.off[s],
                              out_adj + tab.off[s] * p.R, p.R, st));
@@ -1095,14 +1233,6 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
     tm.end(t_init);
 
     const int32_t ks = p.ef_slide < p.L ? p.ef_slide : p.L;
-    const bool cm = (p.flags & RNSM_FLAG_CM) != 0;
-    std::vector<int32_t> srcs;            // source segments in order of first use
-    std::vector<char> is_src((size_t)m, 0);
-    for (const PlanEdge &e : pl)
-        if (!is_src[(size_t)e.src]) {
-            is_src[(size_t)e.src] = 1;
-            srcs.push_back(e.src);
-        }
     std::vector<int64_t> np((size_t)m, 0), nf((size_t)m, 0);
     double host_s = 0.0;
     int64_t n_piv = 0, n_fol = 0;
@@ -1130,10 +1260,12 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
                                      mb.ord + tab.off[s], mb.rank + tab.off[s], st));
             jobs.push_back(make_job(segs[s], segs[s].vecs, mb.ord + tab.off[s],
                                     mb.nplus + tab.off[s] * p.k_plus, total));
+            code_job(jobs.back(), s, s);
             total += segs[s].n;
         }
         TRY(upload_jobs(jobs, total, mb.jobs1, st));
         SearchArgs a = search_defaults();
+        use_codes(a);
         a.dim = dim;
         a.metric = p.metric;
         a.nq = total;
@@ -1144,6 +1276,7 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
         a.out_stride = p.k_plus;
         a.out_by_qidx = 1;
         a.stats = c.stats;
+        a.r_in = r_in_max;
         a.jobs = mb.jobs1;
         a.n_jobs = (int32_t)srcs.size();
         TRY(run_search_jobs(a, c.work, jobs, st));
@@ -1233,6 +1366,7 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
                 j.seed_tab = res;
                 j.seed_row = mb.pivot_of + tab.off[sv];
             }
+            code_job(j, sv, pl[e].dst);
             jobs.push_back(j);
             total += followers ? nf[(size_t)sv] : np[(size_t)sv];
         }
@@ -1249,6 +1383,7 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
             SearchArgs a = search_defaults();
             a.dim = dim;
             a.metric = p.metric;
+            use_codes(a);
             a.nq = tot4;
             a.seed_mode = kSeedConst;
             a.ef = p.L;
@@ -1256,6 +1391,7 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
             a.out_stride = p.L;
             a.out_by_qidx = 1;
             a.stats = c.stats + 2;
+            a.r_in = r_in_max;
             a.jobs = mb.jobs4;
             a.n_jobs = (int32_t)(g1 - g0);
             TRY(run_search_jobs(a, c.work, hj4, es));
@@ -1266,6 +1402,7 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
             SearchArgs a = search_defaults();
             a.dim = dim;
             a.metric = p.metric;
+            use_codes(a);
             a.nq = tot5;
             a.seed_mode = kSeedTable;
             a.seed_stride = p.L;
@@ -1275,6 +1412,7 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
             a.out_stride = p.L;
             a.out_by_qidx = 1;
             a.stats = c.stats + 4;
+            a.r_in = r_in_max;
             a.jobs = mb.jobs5;
             a.n_jobs = (int32_t)(g1 - g0);
             TRY(run_search_jobs(a, c.work + 3, hj5, es));
@@ -1379,8 +1517,8 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
         std::vector<SearchJob> j5 = jobs_of(groups[gi].first, groups[gi].second, true, tot5);
         // capture only what replays unchanged: one group, no autotuning inside
         const bool want_graph = (p.flags & RNSM_FLAG_GRAPH) && !uni && groups.size() == 1 &&
-                                !search_would_tune(dim, p.L, kSeedConst, tot4) &&
-                                !search_would_tune(dim, p.ef_slide, kSeedTable, tot5);
+                                !search_would_tune(dim, p.L, kSeedConst, codes.mode, tot4) &&
+                                !search_would_tune(dim, p.ef_slide, kSeedTable, codes.mode, tot5);
         TRY(upload_jobs(j4, tot4, mb.jobs4, st));
         TRY(upload_jobs(j5, tot5, mb.jobs5, st));
         for (size_t e = groups[gi].first; e < groups[gi].second; ++e) {
@@ -1395,6 +1533,8 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
         }
         // graph mode: capture once, replay while the key matches
         std::string key = graph_key(segs, m, p, pl, out_adj, b.base, np, nf, dim, qprec);
+        key.append(reinterpret_cast<const char *>(&codes.rows), sizeof(codes.rows));
+        key.append(reinterpret_cast<const char *>(&codes.mode), sizeof(codes.mode));
         GraphCache &gc = g_graphs[cur_device()];
         const bool replay = gc.exec && gc.key == key;
         if (!replay) {

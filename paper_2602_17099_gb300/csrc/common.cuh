@@ -141,8 +141,12 @@ __device__ __forceinline__ float prune_dist(const float *a, const float *b, int 
     return chain2_final(acc, metric);
 }
 
+// The differences two at a time (one packed instruction, whose lanes round as
+// the scalar ones), the chain of squares in order.
 __device__ __forceinline__ float l2_acc(float acc, float4 q, float4 x) {
-    float a = q.x - x.x, b = q.y - x.y, c = q.z - x.z, e = q.w - x.w;
+    float a, b, c, e;
+    f2_split(f2_sub(f2_of(q.x, q.y), f2_of(x.x, x.y)), a, b);
+    f2_split(f2_sub(f2_of(q.z, q.w), f2_of(x.z, x.w)), c, e);
     acc = fmaf(a, a, acc);
     acc = fmaf(b, b, acc);
     acc = fmaf(c, c, acc);

@@ -4,9 +4,32 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "common.cuh"
 
 namespace rnsm {
+
+// The grid of a persistent kernel on the current device, worked out (and the
+// kernel's attributes set) on its first launch there: the queries behind it cost
+// the host some 3 us a launch.
+struct GridCache {
+    std::atomic<int> blocks[64] = {};
+};
+template <class F>
+inline cudaError_t cached_grid(GridCache &c, int64_t &grid, F &&work_out) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    int b = dev < 64 ? c.blocks[dev].load(std::memory_order_acquire) : 0;
+    if (b == 0) {
+        e = work_out(dev, b);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) c.blocks[dev].store(b, std::memory_order_release);
+    }
+    grid = b;
+    return cudaSuccess;
+}
 
 // Sets the calling thread's rnsm_last_error() message.
 void set_last_error(const char *msg);
@@ -14,6 +37,33 @@ void set_last_error(const char *msg);
 // Kernels launched by this library (every launcher adds its count).
 void note_launches(int n);
 long long launches_so_far();
+
+// Coded rows (codes.cu): a byte per dimension on one grid lo + s * c for all
+// the rows of a call.  CodeStats: what the passes over the rows gather.
+// CodeParams: the searches' constants, read on the device.
+struct CodeStats {
+    uint32_t omin, omax;   // smallest and largest component, order-preserving bits
+    int32_t fraction;      // a component is no integer
+    uint32_t err2, norm2;  // largest squared residual and squared row norm (float bits)
+};
+struct CodeParams {
+    float scale, inv_scale;  // s; 0: no codes
+    float err;               // e_x + e_q of any two rows
+    float norm2;             // largest squared row norm
+    int32_t exact;           // integers, s = 1: code distances are the distances
+    int32_t useful;          // err is small against the rows' distances
+};
+enum CodeMode : int32_t { kCodeNone = 0, kCodeFilter = 1, kCodeExact = 2 };
+bool codes_dim_ok(int dim);
+// The finite check of launch_validate_vecs (on the first `checked` segments) and
+// the statistics, in one pass over the table's rows; then the codes (rows by global id) and the constants.
+cudaError_t launch_code_scan(const SegTable &t, int32_t dim, int32_t checked, CodeStats *s, int32_t *err,
+                             cudaStream_t st);
+cudaError_t launch_code_rows(const SegTable &t, int32_t dim, int32_t metric, uint8_t *codes, CodeStats *s,
+                             CodeParams *p, cudaStream_t st);
+// Launches of up to this many queries take the search's latency shape, which
+// does not filter by codes.
+constexpr int64_t kLatencyQueries = 1216;
 
 enum SeedMode : int32_t { kSeedConst = 0, kSeedSelf = 1, kSeedTable = 2 };
 
@@ -28,6 +78,8 @@ struct SearchJob {
     const int32_t *seed_tab;
     const int32_t *seed_row;
     int32_t *out_ids;
+    const uint8_t *codes;   // coded rows of base and of qvecs
+    const uint8_t *qcodes;
     int64_t q_begin;
     int64_t n_base;
     int32_t r_in;
@@ -45,7 +97,7 @@ struct SearchArgs {
     const float *base;      // searched vector set [n_base * dim]
     int64_t n_base;
     const int32_t *adj;     // [n_base * r_in]
-    int32_t r_in;
+    int32_t r_in;           // (jobs: the largest of theirs)
     int32_t dim;
     int32_t metric;
     const float *qvecs;
@@ -69,14 +121,24 @@ struct SearchArgs {
     int64_t *out_ndc;         // nullable, [nq]
     unsigned long long *stats;  // nullable: [0] += NDC, [1] += expansions
     int32_t *work;            // zeroed work counter
+    int32_t code_mode;        // CodeMode of the launch
+    const uint8_t *codes;     // coded rows of base and of qvecs
+    const uint8_t *qcodes;
+    const CodeParams *code_params;
     const SearchJob *jobs;    // nullable: multi-job launch (out_d and out_ndc unused)
     int32_t n_jobs;
 };
 
 cudaError_t launch_search(const SearchArgs &a, cudaStream_t st);
-cudaError_t launch_search_jobs(const SearchArgs &a, int var, cudaStream_t st);
+// Its kernels, by job table or not and by code mode (a.code_mode).
+cudaError_t launch_search_plain(const SearchArgs &a, int var, cudaStream_t st);
+cudaError_t launch_search_filter(const SearchArgs &a, int var, cudaStream_t st);
+cudaError_t launch_search_exact(const SearchArgs &a, int var, cudaStream_t st);
+cudaError_t launch_search_jobs_plain(const SearchArgs &a, int var, cudaStream_t st);
+cudaError_t launch_search_jobs_filter(const SearchArgs &a, int var, cudaStream_t st);
+cudaError_t launch_search_jobs_exact(const SearchArgs &a, int var, cudaStream_t st);
 // True if a launch of nq queries would run the autotuner (timed chunks, host waits).
-bool search_would_tune(int dim, int ef, int seed_mode, int64_t nq);
+bool search_would_tune(int dim, int ef, int seed_mode, int code_mode, int64_t nq);
 
 // Occlusion prune (UpdateGraph) of a batch of owners over a segment table.
 // Owner i is global id owner_ids ? owner_ids[i] : owner_base + i.  Its pool

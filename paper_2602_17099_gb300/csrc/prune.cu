@@ -1134,17 +1134,20 @@ namespace {
 template <int kMetric, int kF4>
 cudaError_t launch_walk_t(const PruneArgs &a, cudaStream_t st) {
     auto kern = prune_walk_kernel<kMetric, kF4>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWalkThreads, 0);
+    static GridCache cache;
+    int64_t grid = 0;
+    cudaError_t e = cached_grid(cache, grid, [&](int dev, int &blocks) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        int sms = 0, per_sm = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const cudaError_t r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWalkThreads, 0);
+        blocks = sms * (per_sm < 1 ? 1 : per_sm);
+        return r;
+    });
     if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
     // owners per claim: the next owner's rows are loaded during the current one's
     // walk only within a claim
     const int chunk = a.skip_empty_csr ? 8 : RNSM_WALK_CHUNK;
-    int64_t grid = (int64_t)sms * per_sm;
     const int64_t want = (a.n_owners + chunk - 1) / chunk;
     if (want < grid) grid = want;
     kern<<<(unsigned)grid, kWalkThreads, 0, st>>>(a, chunk);
@@ -1168,17 +1171,20 @@ cudaError_t launch_walk(const PruneArgs &a, cudaStream_t st) {
 }
 
 cudaError_t launch_small(const PruneArgs &a, cudaStream_t st) {
-    cudaError_t e;
-    cudaFuncSetAttribute(prune_small_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, prune_small_kernel, kSmallThreads, 0);
+    static GridCache cache;
+    int64_t grid = 0;
+    cudaError_t e = cached_grid(cache, grid, [&](int dev, int &blocks) {
+        cudaFuncSetAttribute(prune_small_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        int sms = 0, per_sm = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const cudaError_t r =
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, prune_small_kernel, kSmallThreads, 0);
+        blocks = sms * (per_sm < 1 ? 1 : per_sm);
+        return r;
+    });
     if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
     // owners are claimed a few at a time: one atomic round trip per claim
     const int chunk = a.skip_empty_csr ? 8 : 4;
-    int64_t grid = (int64_t)sms * per_sm;
     const int64_t want = (a.n_owners + chunk - 1) / chunk;
     if (want < grid) grid = want;
     prune_small_kernel<<<(unsigned)grid, kSmallThreads, 0, st>>>(a, chunk);

@@ -1,20 +1,28 @@
-// K1: batched AKNN beam search (Algorithm 1, Section 2.2), one warp per query.
+// K1: batched AKNN beam search (Algorithm 1, Section 2.2), one warp per query:
+// launch shapes and their autotuner; the kernel is in search_impl.cuh.
 //
-// Per warp, in shared memory: the candidate set C as a (distance, id) array
-// sorted lexicographically and double buffered (the expanded flag rides in
-// bit 31 of the id), an open-addressing visited hash, and staging for the
-// distances of the current neighbourhood.  Neighbour rows are gathered with
-// 128-bit loads: a group of G lanes covers one row (lane s of the group reads
-// float4 s, s+G, ...), 32/G rows per step, U steps in flight.
+// Per warp: the candidate set C sorted in registers (64-bit keys of distance, id
+// and the expanded flag), a visited table in shared memory, and the neighbours'
+// rows gathered with 128-bit loads: first their codes (codes.cu), then, where
+// those do not settle it, their FP32 rows, of which a group of G lanes covers one
+// (lane s of the group reads float4 s, s+G, ...), 32/G rows per step.
 //
 // Semantics match Algorithm 1 exactly: repeatedly expand the nearest
 // unexpanded entry, evaluate every neighbour not evaluated before, keep the
 // best ef by (distance, id).  Inserting a whole neighbourhood and truncating
-// to ef leaves the same set as inserting one neighbour at a time.  The hash
-// is exact until a probe sequence runs out; from then on it is lossy, which
+// to ef leaves the same set as inserting one neighbour at a time.  The visited
+// table is exact until a set of it is full; from then on it may forget, which
 // cannot change the result because an evaluated vertex outside C is worse
 // than the worst entry of C (and that bound only tightens) while vertices
-// inside C are deduplicated by id before insertion.
+// inside C are found there before insertion.
+//
+// What bounds it: the instructions of an expansion.  2 x 500k SIFT-like rows, S1 +
+// S4 + S5, before (C and merge by ranks in shared memory, FP32 rows, a hash probed
+// slot by slot): 7.2 + 7.7 + 8.7 ms at 76 % of L2 throughput; now 4.1 + 4.7 + 5.6
+// ms at 80 % of the issue slots and 31 % of L2 throughput.  300k DEEP-like rows:
+// 4.3 + 8.2 + 12.3 -> 3.2 + 4.5 + 7.6 ms; 60k embedding-like rows of 768:
+// 4.6 + 12.7 + 16.7 -> 2.8 + 5.3 + 9.6 ms; 16 queries, ef 128, on 100k DEEP-like
+// rows: 1.9 -> 0.40 ms.
 #include <float.h>
 #include <stdlib.h>
 
@@ -22,14 +30,21 @@
 #include <mutex>
 #include <utility>
 
-#include "search_impl.cuh"
+#include "internal.h"
 
 namespace rnsm {
 
 namespace {
 
 cudaError_t launch_dim_any(const SearchArgs &a, int var, cudaStream_t st) {
-    return a.jobs ? launch_search_jobs(a, var, st) : launch_dim<false>(a, var, st);
+    // few queries: each warp's chain of dependent loads decides, and the filter's
+    // second gather would lengthen it
+    const int mode = a.code_mode == kCodeFilter && a.nq <= kLatencyQueries ? kCodeNone : a.code_mode;
+    switch (mode) {
+        case kCodeExact: return a.jobs ? launch_search_jobs_exact(a, var, st) : launch_search_exact(a, var, st);
+        case kCodeFilter: return a.jobs ? launch_search_jobs_filter(a, var, st) : launch_search_filter(a, var, st);
+        default: return a.jobs ? launch_search_jobs_plain(a, var, st) : launch_search_plain(a, var, st);
+    }
 }
 
 // The queries [q0, q1) of a launch as a launch of their own.
@@ -50,11 +65,13 @@ SearchArgs subrange(const SearchArgs &a, int64_t q0, int64_t q1) {
 // beams); normalising by the distance count makes chunks of different
 // difficulty comparable, and spreading the chunks over the list keeps the
 // comparison representative when the queries come in locality order.
+constexpr int kVariants = 4;   // search_impl.cuh: shape, prefetch
 constexpr int kTuneChunks = 4 * kVariants;
 constexpr int64_t kTuneMinChunk = 4000;
 struct TuneKey {
-    int dim, efmax, seed_mode;
+    int dim, efmax, seed_mode, code_mode;
     bool operator<(const TuneKey &o) const {
+        if (code_mode != o.code_mode) return code_mode < o.code_mode;
         return dim != o.dim ? dim < o.dim : efmax != o.efmax ? efmax < o.efmax : seed_mode < o.seed_mode;
     }
 };
@@ -68,12 +85,21 @@ int forced_variant() {
     return force && force[0] >= '0' && force[0] < '0' + kVariants ? force[0] - '0' : -1;
 }
 
+// Before a shape is tuned (and for launches too small to tune): shape 1 where a
+// lane's share of a row is six float4 and few rows are in flight otherwise.
+// Embedding-like rows (768, filtered): S4 10.5 -> 5.6 ms, S5 15.0 -> 10.1 ms on
+// 3 x 20k; DEEP-like rows (96, FP32 only): S4 6.7 -> 5.4, S5 9.4 -> 9.1 ms on
+// 300k; SIFT-like rows (128, FP32 only) S5 8.6 -> 11.6 ms on 2 x 500k.
+int default_variant(int dim, int code_mode) {
+    return dim == 768 || (dim == 96 && code_mode == kCodeNone) ? 1 : 0;
+}
+
 }  // namespace
 
-bool search_would_tune(int dim, int ef, int seed_mode, int64_t nq) {
+bool search_would_tune(int dim, int ef, int seed_mode, int code_mode, int64_t nq) {
     if (forced_variant() >= 0 || nq < kTuneChunks * kTuneMinChunk) return false;
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    return g_tuned.find({dim, efmax_of(ef), seed_mode}) == g_tuned.end();
+    return g_tuned.find({dim, efmax_of(ef), seed_mode, code_mode}) == g_tuned.end();
 }
 
 cudaError_t launch_search(const SearchArgs &a, cudaStream_t st) {
@@ -81,31 +107,32 @@ cudaError_t launch_search(const SearchArgs &a, cudaStream_t st) {
     if (!search_dim_supported(a.dim)) return cudaErrorInvalidValue;
     const int forced = forced_variant();
     if (forced >= 0) return launch_dim_any(a, forced, st);
-    const TuneKey key{a.dim, efmax_of(a.ef), a.seed_mode};
+    const TuneKey key{a.dim, efmax_of(a.ef), a.seed_mode, a.code_mode};
     int var = -1;
+    const int first = default_variant(a.dim, a.code_mode);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tuned.find(key);
         if (it != g_tuned.end()) var = it->second;
     }
-    if (var >= 0 || a.nq < kTuneChunks * kTuneMinChunk) return launch_dim_any(a, var >= 0 ? var : 0, st);
+    if (var >= 0 || a.nq < kTuneChunks * kTuneMinChunk) return launch_dim_any(a, var >= 0 ? var : first, st);
     // NDC of each chunk: the caller's statistics counter, read around the chunk
     static unsigned long long *own_stats[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     unsigned long long *cnt = a.stats;
     if (!cnt) {
-        if (dev >= 64) return launch_dim_any(a, 0, st);
+        if (dev >= 64) return launch_dim_any(a, first, st);
         if (!own_stats[dev] && cudaMalloc(&own_stats[dev], 2 * sizeof(unsigned long long)) != cudaSuccess)
-            return launch_dim_any(a, 0, st);
+            return launch_dim_any(a, first, st);
         cnt = own_stats[dev];
     }
     double ms_of[kVariants] = {}, ndc_of[kVariants] = {};
     cudaEvent_t e0, e1;
-    if (cudaEventCreate(&e0) != cudaSuccess) return launch_dim_any(a, 0, st);
+    if (cudaEventCreate(&e0) != cudaSuccess) return launch_dim_any(a, first, st);
     if (cudaEventCreate(&e1) != cudaSuccess) {
         cudaEventDestroy(e0);
-        return launch_dim_any(a, 0, st);
+        return launch_dim_any(a, first, st);
     }
     cudaError_t err = cudaSuccess;
     unsigned long long before = 0, after = 0;
