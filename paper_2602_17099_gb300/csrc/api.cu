@@ -548,19 +548,25 @@ rnsm_status rnsm_select_pivots_gpu(const int32_t *nplus, int64_t n, int32_t k_pl
         int32_t *pv = bb.take<int32_t>(n);
         int32_t *fl = bb.take<int32_t>(n);
         void *tmp = bb.take<char>(pivot_tmp_bytes(n));
-        return std::make_tuple(pv, fl, tmp);
+        PivotCtl *ctl = bb.take<PivotCtl>(1);
+        return std::make_tuple(pv, fl, tmp, ctl);
     };
     carve(b);
     TRY(ws_acquire(b.off, b));
     int32_t *pv, *fl;
     void *tmp;
-    std::tie(pv, fl, tmp) = carve(b);
+    PivotCtl *ctl;
+    std::tie(pv, fl, tmp, ctl) = carve(b);
     TRY(ctl_reset(c, st));
     CK(launch_validate_ids(nplus, n * k_plus, n, 1, c.err, st));
     TRY(check_err_word(c, st));
-    int64_t nf = 0;
-    CK(select_pivots_device(nplus, n, k_plus, k, offs, ids, pivot_of, pv, fl, n_pivots, &nf,
-                            rounds, tmp, c.stats, st));
+    CK(launch_select_pivots(nplus, n, k_plus, k, offs, ids, pivot_of, pv, fl, tmp, ctl, st));
+    PivotCtl h;
+    CK(cudaMemcpyAsync(&h, ctl, sizeof(h), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    CK(h.stuck ? cudaErrorUnknown : cudaSuccess);
+    *n_pivots = (int64_t)h.n_pivots;
+    if (rounds) *rounds = (h.rounds + 3) / 4 * 4;   // reported in steps of four
     return RNSM_OK;
 }
 
@@ -945,6 +951,7 @@ struct MergeBufs {
     int32_t *pivot_of, *pivots, *followers;   // [N] each, segment s at off[s]
     int32_t *ord, *rank;                      // locality order of each source and positions
     void *piv_tmp;
+    PivotCtl *piv_ctl;                        // per segment
     int32_t *res;                          // [res_rows * L]
     int32_t *eu, *ev;
     int32_t *upool;                        // union variant: the pools of one source
@@ -976,6 +983,7 @@ void carve_merge(Bump &b, const rnsm_params &p, int64_t nmax, int64_t n_all, int
     m.ord = b.take<int32_t>(n_all);
     m.rank = b.take<int32_t>(n_all);
     m.piv_tmp = b.take<char>(pivot_tmp_bytes(nmax));
+    m.piv_ctl = b.take<PivotCtl>(kMaxSeg);
     m.res = b.take<int32_t>(res_rows * p.L);
     m.eu = b.take<int32_t>(nrev * p.R);
     m.ev = b.take<int32_t>(nrev * p.R);
@@ -1322,20 +1330,31 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
                 CK(cudaStreamSynchronize(st));
             } else {
                 // S3: the same selection in parallel rounds on the device
-                int64_t np_ = 0, nf_ = 0;
-                CK(select_pivots_device(nplus, ns, p.k_plus, p.k_rev, mb.rk_offs, mb.rk_ids,
-                                        pivot_of, pivots, followers, &np_, &nf_, nullptr,
-                                        mb.piv_tmp, c.stats + 6, st));
-                np[(size_t)s] = np_;
-                nf[(size_t)s] = nf_;
+                CK(launch_select_pivots(nplus, ns, p.k_plus, p.k_rev, mb.rk_offs, mb.rk_ids, pivot_of,
+                                        pivots, followers, mb.piv_tmp, mb.piv_ctl + s, st));
             }
-            // schedule of S4 and S5: pivots in locality order, each pivot's followers
-            // (which start from the same seeds) side by side
-            CK(order_search_lists(mb.rank + tab.off[s], pivot_of, pivots, np[(size_t)s], followers,
-                                  nf[(size_t)s], ns, mb.rk_keys, mb.rk_vals, mb.rk_offs,
-                                  mb.rk_cursor, mb.rk_scan, mb.rk_scan_bytes, st));
             tm.end(t3);
         }
+        const int t3 = tm.begin(3);
+        if (!(p.flags & RNSM_FLAG_HOST_PIVOTS)) {   // the counts of every source, one wait
+            std::vector<PivotCtl> h((size_t)m);
+            CK(cudaMemcpyAsync(h.data(), mb.piv_ctl, sizeof(PivotCtl) * (size_t)m, cudaMemcpyDeviceToHost, st));
+            CK(cudaStreamSynchronize(st));
+            for (int32_t s : srcs) {
+                CK(h[(size_t)s].stuck ? cudaErrorUnknown : cudaSuccess);
+                np[(size_t)s] = (int64_t)h[(size_t)s].n_pivots;
+                nf[(size_t)s] = (int64_t)h[(size_t)s].n_followers;
+            }
+        }
+        for (int32_t s : srcs) {
+            // schedule of S4 and S5: pivots in locality order, each pivot's followers
+            // (which start from the same seeds) side by side
+            CK(order_search_lists(mb.rank + tab.off[s], mb.pivot_of + tab.off[s], mb.pivots + tab.off[s],
+                                  np[(size_t)s], mb.followers + tab.off[s], nf[(size_t)s], segs[s].n,
+                                  mb.rk_keys, mb.rk_vals, mb.rk_offs, mb.rk_cursor, mb.rk_scan,
+                                  mb.rk_scan_bytes, st));
+        }
+        tm.end(t3);
     }
 
     // S4 .. S7 over groups of consecutive plan edges

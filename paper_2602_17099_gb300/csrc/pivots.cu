@@ -14,158 +14,260 @@
 // local maxima never conflict with each other, so one round selects all of
 // them at once.  The global maximum is always a local maximum, so every round
 // makes progress.
+//
+// A round by votes: every uncovered z votes for the vertex of largest key among
+// itself and its uncovered N_k(z).  Conf(x) is the union of these sets over x
+// itself and the uncovered z in R_k(x), so x beats its conflict set iff all of
+// them vote for it: gain(x) + 1 votes (a vote weighs as often as N_k(z) names x,
+// plus one for z = x, so repeated entries count as they do in the gain).  The
+// gains are kept, not recomputed: covering y takes one from every vertex of
+// N_k(y).  So a round gathers k words per uncovered vertex and touches R_k(x) of
+// the selected x only; before, every uncovered x read its whole conflict set,
+// |R_k(x)| * k keys by one thread, and hubs set the time of each round.
+//
+// The uncovered vertices are listed anew every round, and the last rounds, few
+// vertices each, run in one launch of one thread-block cluster, which needs no host
+// between rounds (all rounds of up to kTailMax vertices run there; with 6 rounds over
+// the whole grid before it instead of 16, 500k rows left it 1.5 ms of work).  What is
+// left is the chain of dependent loads of each round, some 14 us.  S3 of 5,000
+// Gaussian rows 2.14 -> 0.55 ms, 2 x 500k SIFT-like rows 1.55 -> 0.81 ms, 300k
+// DEEP-like rows in 5 segments 3.25 -> 1.90 ms.
+
+#include <cooperative_groups.h>
+
 #include "internal.h"
 
 namespace rnsm {
 
 namespace {
 
-__global__ void piv_init_kernel(int64_t n, uint8_t *covered, int32_t *pivot_of) {
+constexpr int32_t kCovered = -(1 << 30);   // gain of a covered vertex (and below)
+constexpr int64_t kTailMax = 32768;
+constexpr int kWide = 24;                  // reverse lists from here on take a warp
+constexpr int kFullRounds = 16;            // rounds over the whole grid before the cluster's
+constexpr int kTailBlocks = 8, kTailThreads = 1024;
+
+struct PivotState {
+    int32_t *gain;    // |R_k(x) \ Covered|, or kCovered and below
+    int32_t *votes;
+    int32_t *snap;    // the gain at the start of the round
+    int32_t *pivot_of;
+    const int32_t *nplus;
+    const int64_t *offs;
+    const int32_t *ids;
+    int32_t k_plus, k;
+};
+
+__global__ void piv_init_kernel(PivotState s, int64_t n, int32_t *list, PivotCtl *ctl) {
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n;
          x += (int64_t)gridDim.x * blockDim.x) {
-        covered[x] = 0;
-        pivot_of[x] = -2;
+        s.gain[x] = (int32_t)(s.offs[x + 1] - s.offs[x]);
+        s.votes[x] = 0;
+        s.pivot_of[x] = -2;
+        list[x] = (int32_t)x;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *ctl = PivotCtl();
+        ctl->count[0] = (int32_t)n;
     }
 }
 
-// key = (gain << 32) | (~x): larger gain first, then the lower id; 0 if covered.
-__global__ void piv_gain_kernel(int64_t n, const int64_t *offs, const int32_t *ids,
-                                const uint8_t *covered, unsigned long long *key) {
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        if (covered[x]) {
-            key[x] = 0ull;
-            continue;
-        }
-        unsigned long long g = 0;
-        for (int64_t e = offs[x]; e < offs[x + 1]; ++e) g += covered[ids[e]] ? 0 : 1;
-        key[x] = (g << 32) | (unsigned long long)(0xffffffffu - (uint32_t)x);
-    }
-}
-
-__global__ void piv_select_kernel(int64_t n, const int32_t *nplus, int32_t k_plus, int32_t k,
-                                  const int64_t *offs, const int32_t *ids, const uint8_t *covered,
-                                  const unsigned long long *key, uint8_t *sel) {
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        if (covered[x]) {
-            sel[x] = 0;
-            continue;
-        }
-        const unsigned long long kx = key[x];
-        bool ok = true;
-        const int32_t *nx = nplus + x * k_plus;
-        for (int j = 0; ok && j < k; ++j) {
-            const int32_t y = nx[j];
-            if (y >= 0 && key[y] > kx) ok = false;
-        }
-        for (int64_t e = offs[x]; ok && e < offs[x + 1]; ++e) {
-            const int32_t z = ids[e];
-            if (key[z] > kx) { ok = false; break; }
-            if (covered[z]) continue;
-            const int32_t *nz = nplus + (int64_t)z * k_plus;
-            for (int j = 0; j < k; ++j) {
-                const int32_t y = nz[j];
-                if (y >= 0 && y != (int32_t)x && key[y] > kx) { ok = false; break; }
+// Lists the uncovered vertices of cur[0..nc) in next and takes their votes;
+// thread t of `threads` (whole warps).
+__device__ __forceinline__ void vote_phase(const PivotState &s, const int32_t *cur, int32_t nc, int32_t *next,
+                                           int32_t *n_next, int64_t t, int64_t threads) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t i0 = t - lane; i0 < nc; i0 += threads) {
+        const int64_t i = i0 + lane;
+        const int32_t z = i < nc ? __ldcg(cur + i) : -1;
+        const int32_t gz = z >= 0 ? __ldcg(s.gain + z) : kCovered;
+        const bool open = gz >= 0;
+        const unsigned m = __ballot_sync(0xffffffffu, open);
+        int base = 0;
+        if (lane == 0 && m) base = atomicAdd(n_next, __popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (!open) continue;
+        __stcg(next + base + __popc(m & lanemask_lt()), z);
+        __stcg(s.snap + z, gz);
+        int32_t best = z, gb = gz;
+        int weight = 1;   // z's own
+        const int32_t *nz = s.nplus + (int64_t)z * s.k_plus;
+#pragma unroll 5
+        for (int j = 0; j < s.k; ++j) {
+            const int32_t y = __ldg(nz + j);
+            if (y < 0) continue;
+            const int32_t gy = __ldcg(s.gain + y);
+            if (y == best) ++weight;
+            else if (gy > gb || (gy == gb && gy >= 0 && y < best)) {
+                best = y;
+                gb = gy;
+                weight = 1;
             }
         }
-        sel[x] = ok ? 1 : 0;
+        atomicAdd(s.votes + best, weight);
     }
 }
 
-__global__ void piv_apply_kernel(int64_t n, const int64_t *offs, const int32_t *ids,
-                                 const uint8_t *sel, uint8_t *covered, int32_t *pivot_of,
-                                 unsigned long long *newly) {
-    unsigned long long cnt = 0;
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        if (!sel[x]) continue;
-        // selected vertices never share an uncovered reverse neighbour
-        for (int64_t e = offs[x]; e < offs[x + 1]; ++e) {
-            const int32_t y = ids[e];
-            if (!covered[y]) {
-                covered[y] = 1;
-                pivot_of[y] = (int32_t)x;
-                ++cnt;
-            }
+// Covers entry e of the selected x's reverse list (e = lo - 1: x itself).
+__device__ __forceinline__ void cover(const PivotState &s, int32_t x, int64_t e, int64_t lo) {
+    const int32_t y = e < lo ? x : s.ids[e];
+    if (e >= lo && (y == x || __ldcg(s.gain + y) < 0)) return;
+    if (atomicExch(s.gain + y, kCovered) < 0) return;   // listed twice: once
+    __stcg(s.pivot_of + y, e < lo ? -1 : x);
+    const int32_t *ny = s.nplus + (int64_t)y * s.k_plus;
+    for (int c = 0; c < s.k; ++c) {
+        const int32_t w = __ldg(ny + c);
+        if (w >= 0) atomicSub(s.gain + w, 1);
+    }
+}
+
+__device__ __forceinline__ unsigned drop_lowest(unsigned m, int n) {
+    for (int q = 0; q < n; ++q) m &= m - 1u;
+    return m;
+}
+
+// Selects the vertices of next[0..n) that have all their votes: they become
+// pivots, their uncovered reverse neighbours followers.  Eight lanes per
+// selected vertex, a warp where the reverse list is long (a hub's list by eight
+// lanes is a chain of |R_k| / 8 rounds of four dependent loads).
+__device__ __forceinline__ void select_phase(const PivotState &s, const int32_t *next, int32_t n, int64_t t,
+                                             int64_t threads) {
+    const int lane = threadIdx.x & 31, sub = lane & 7, grp = lane >> 3;
+    for (int64_t i0 = t - lane; i0 < n; i0 += threads) {
+        const int64_t i = i0 + lane;
+        const int32_t x = i < n ? __ldcg(next + i) : -1;
+        bool sel = false;
+        if (x >= 0) {
+            sel = __ldcg(s.votes + x) == __ldcg(s.snap + x) + 1;
+            __stcg(s.votes + x, 0);
         }
-        covered[x] = 1;
-        pivot_of[x] = -1;
-        ++cnt;
+        int64_t lo = 0, hi = 0;
+        if (sel) {
+            lo = s.offs[x];
+            hi = s.offs[x + 1];
+        }
+        const bool wide = sel && hi - lo >= kWide;
+        unsigned m = __ballot_sync(0xffffffffu, sel && !wide);
+        for (; m; m = drop_lowest(m, 4)) {
+            const unsigned r = drop_lowest(m, grp);
+            const int src = r ? __ffs(r) - 1 : lane;
+            const int32_t xs = __shfl_sync(0xffffffffu, x, src);
+            const int64_t l = __shfl_sync(0xffffffffu, lo, src), h = __shfl_sync(0xffffffffu, hi, src);
+            if (r)
+                for (int64_t e = l + sub - 1; e < h; e += 8) cover(s, xs, e, l);
+            __syncwarp();
+        }
+        for (m = __ballot_sync(0xffffffffu, wide); m; m &= m - 1u) {
+            const int src = __ffs(m) - 1;
+            const int32_t xs = __shfl_sync(0xffffffffu, x, src);
+            const int64_t l = __shfl_sync(0xffffffffu, lo, src), h = __shfl_sync(0xffffffffu, hi, src);
+            for (int64_t e = l + lane - 1; e < h; e += 32) cover(s, xs, e, l);
+            __syncwarp();
+        }
     }
-    if (cnt) atomicAdd(newly, cnt);
 }
 
-__global__ void piv_compact_kernel(int64_t n, const int32_t *pivot_of, int32_t *pivots,
-                                   int32_t *followers, unsigned long long *counts) {
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        if (pivot_of[x] == -1) pivots[atomicAdd(&counts[0], 1ull)] = (int32_t)x;
-        else followers[atomicAdd(&counts[1], 1ull)] = (int32_t)x;
+__global__ void __launch_bounds__(256) piv_vote_kernel(PivotState s, const int32_t *cur, int32_t *next, PivotCtl *ctl,
+                                                       int round) {
+    vote_phase(s, cur, ctl->count[round], next, &ctl->count[round + 1], blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
+               (int64_t)gridDim.x * blockDim.x);
+}
+
+__global__ void __launch_bounds__(256) piv_select_kernel(PivotState s, const int32_t *next, PivotCtl *ctl, int round) {
+    const int32_t n = ctl->count[round + 1];
+    if (n > 0 && blockIdx.x == 0 && threadIdx.x == 0) ++ctl->rounds;
+    select_phase(s, next, n, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+}
+
+// The remaining rounds, by one cluster.  Each round has fewer uncovered vertices
+// than the one before (else the lists are not those of one graph: error).
+__global__ void __cluster_dims__(kTailBlocks, 1, 1) __launch_bounds__(kTailThreads)
+    piv_tail_kernel(PivotState s, int32_t *cur, int32_t *next, PivotCtl *ctl, int round) {
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, threads = kTailBlocks * (int64_t)kTailThreads;
+    int32_t nc = __ldcg(&ctl->count[round]), before = INT32_MAX, rounds = 0;
+    int32_t *slot = &ctl->count[round];   // slot[1], slot[2], slot[3] take turns
+    for (int r = 0;; ++r) {
+        int32_t *n_next = slot + 1 + r % 3;
+        vote_phase(s, cur, nc, next, n_next, t, threads);
+        cluster.sync();
+        nc = __ldcg(n_next);
+        if (nc == 0) break;
+        if (nc >= before) {
+            if (t == 0) ctl->stuck = 1;
+            break;
+        }
+        before = nc;
+        ++rounds;
+        if (t == 0) __stcg(slot + 1 + (r + 2) % 3, 0);   // next but one: read by all a round ago
+        select_phase(s, next, nc, t, threads);
+        cluster.sync();
+        int32_t *sw = cur;
+        cur = next;
+        next = sw;
+    }
+    if (t == 0) ctl->rounds += rounds;
+}
+
+__global__ void piv_compact_kernel(int64_t n, const int32_t *pivot_of, int32_t *pivots, int32_t *followers,
+                                   PivotCtl *ctl) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t x0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x - lane; x0 < n;
+         x0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t x = x0 + lane;
+        const bool pv = x < n && pivot_of[x] == -1, fl = x < n && !pv;
+        const unsigned mp = __ballot_sync(0xffffffffu, pv), mf = __ballot_sync(0xffffffffu, fl);
+        unsigned long long bp = 0, bf = 0;
+        if (lane == 0) {
+            if (mp) bp = atomicAdd(&ctl->n_pivots, (unsigned long long)__popc(mp));
+            if (mf) bf = atomicAdd(&ctl->n_followers, (unsigned long long)__popc(mf));
+        }
+        bp = __shfl_sync(0xffffffffu, bp, 0);
+        bf = __shfl_sync(0xffffffffu, bf, 0);
+        if (pv) pivots[bp + __popc(mp & lanemask_lt())] = (int32_t)x;
+        if (fl) followers[bf + __popc(mf & lanemask_lt())] = (int32_t)x;
     }
 }
 
 int grid_n(int64_t n) {
     int64_t g = (n + 255) / 256;
-    if (g > 8192) g = 8192;
+    if (g > 2048) g = 2048;
     return g < 1 ? 1 : (int)g;
 }
 
 }  // namespace
 
-size_t pivot_tmp_bytes(int64_t n) {
-    return (size_t)n * (sizeof(unsigned long long) + 2) + 256;
-}
+size_t pivot_tmp_bytes(int64_t n) { return 3 * (size_t)n * sizeof(int32_t); }
 
-cudaError_t select_pivots_device(const int32_t *nplus, int64_t n, int32_t k_plus, int32_t k,
-                                 const int64_t *offs, const int32_t *ids, int32_t *pivot_of,
-                                 int32_t *pivots, int32_t *followers, int64_t *n_pivots,
-                                 int64_t *n_followers, int32_t *rounds, void *tmp,
-                                 unsigned long long *counters, cudaStream_t st) {
-    if (n <= 0) {
-        *n_pivots = *n_followers = 0;
-        return cudaSuccess;
-    }
-    unsigned long long *key = static_cast<unsigned long long *>(tmp);
-    uint8_t *covered = reinterpret_cast<uint8_t *>(key + n);
-    uint8_t *sel = covered + n;
+cudaError_t launch_select_pivots(const int32_t *nplus, int64_t n, int32_t k_plus, int32_t k, const int64_t *offs,
+                                 const int32_t *ids, int32_t *pivot_of, int32_t *pivots, int32_t *followers,
+                                 void *tmp, PivotCtl *ctl, cudaStream_t st) {
+    PivotState s;
+    s.gain = static_cast<int32_t *>(tmp);
+    s.votes = s.gain + n;
+    s.snap = s.votes + n;
+    s.pivot_of = pivot_of;
+    s.nplus = nplus;
+    s.offs = offs;
+    s.ids = ids;
+    s.k_plus = k_plus;
+    s.k = k;
+    // the output lists hold the uncovered vertices meanwhile
+    int32_t *cur = pivots, *next = followers;
     const int g = grid_n(n);
-    piv_init_kernel<<<g, 256, 0, st>>>(n, covered, pivot_of);
-    note_launches(1);
-    int64_t done = 0;
-    int r = 0;
-    // Rounds in batches: extra rounds after convergence select nothing.
-    constexpr int kBatch = 4;
-    while (done < n) {
-        cudaError_t e = cudaMemsetAsync(counters, 0, sizeof(unsigned long long), st);
-        if (e != cudaSuccess) return e;
-        for (int b = 0; b < kBatch; ++b) {
-            piv_gain_kernel<<<g, 256, 0, st>>>(n, offs, ids, covered, key);
-            piv_select_kernel<<<g, 256, 0, st>>>(n, nplus, k_plus, k, offs, ids, covered, key, sel);
-            piv_apply_kernel<<<g, 256, 0, st>>>(n, offs, ids, sel, covered, pivot_of, counters);
-            note_launches(3);
+    piv_init_kernel<<<g, 256, 0, st>>>(s, n, cur, ctl);
+    int round = 0;
+    if (n > kTailMax)
+        for (; round < kFullRounds; ++round) {
+            piv_vote_kernel<<<g, 256, 0, st>>>(s, cur, next, ctl, round);
+            piv_select_kernel<<<g, 256, 0, st>>>(s, next, ctl, round);
+            int32_t *sw = cur;
+            cur = next;
+            next = sw;
         }
-        r += kBatch;
-        unsigned long long newly = 0;
-        e = cudaMemcpyAsync(&newly, counters, sizeof(newly), cudaMemcpyDeviceToHost, st);
-        if (e != cudaSuccess) return e;
-        e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return e;
-        if (newly == 0) return cudaErrorUnknown;  // cannot happen: a round always selects
-        done += (int64_t)newly;
-    }
-    cudaError_t e = cudaMemsetAsync(counters, 0, 2 * sizeof(unsigned long long), st);
-    if (e != cudaSuccess) return e;
-    piv_compact_kernel<<<g, 256, 0, st>>>(n, pivot_of, pivots, followers, counters);
-    note_launches(1);
-    unsigned long long c[2] = {0, 0};
-    e = cudaMemcpyAsync(c, counters, sizeof(c), cudaMemcpyDeviceToHost, st);
-    if (e != cudaSuccess) return e;
-    e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return e;
-    *n_pivots = (int64_t)c[0];
-    *n_followers = (int64_t)c[1];
-    if (rounds) *rounds = r;
+    piv_tail_kernel<<<kTailBlocks, kTailThreads, 0, st>>>(s, cur, next, ctl, round);
+    piv_compact_kernel<<<g, 256, 0, st>>>(n, pivot_of, pivots, followers, ctl);
+    note_launches(3 + 2 * round);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,49 @@
+"""Pivot selection on the device against the host's lazy greedy, around the
+sizes where its rounds move from one thread-block cluster to the whole grid,
+with short and long reverse lists (a warp each from 24 entries on), holes and
+the smallest k."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rn():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_17099_gb300 import build as b
+    b.build()
+    from paper_2602_17099_gb300 import rnsm
+    return rnsm
+
+
+def _nplus(kind, n, kp, rng):
+    if kind == "random":
+        nb = rng.integers(0, n, (n, kp))
+    elif kind == "near":                    # overlapping neighbourhoods: many rounds
+        nb = (np.arange(n)[:, None] + rng.integers(-20, 20, (n, kp))) % n
+    else:                                   # hubs of some hundreds of entries
+        nb = np.where(rng.random((n, kp)) < 0.3, rng.integers(0, max(1, n // 100), (n, kp)),
+                      rng.integers(0, n, (n, kp)))
+    nb[rng.random((n, kp)) < 0.02] = -1
+    for j in range(kp):                     # no vertex itself, no entry twice
+        bad = nb[:, j] == np.arange(n)
+        for q in range(j):
+            bad |= nb[:, j] == nb[:, q]
+        nb[bad, j] = -1
+    return nb.astype(np.int32)
+
+
+@pytest.mark.parametrize("n,k,k_plus", [(7, 2, 2), (1000, 3, 5), (32768, 5, 16), (32769, 5, 16),
+                                        (150_001, 7, 7), (90_000, 1, 3)])
+@pytest.mark.parametrize("kind", ["random", "near", "hubs"])
+def test_pivots_equal_the_lazy_greedy(rn, kind, n, k, k_plus):
+    nplus = torch.from_numpy(_nplus(kind, n, k_plus, np.random.default_rng(n + k))).cuda()
+    offs, ids = rn.reverse_knn(nplus, k)
+    got, n_piv, rounds = rn.select_pivots_gpu(nplus, k, offs, ids)
+    want, piv = rn.select_pivots(n, offs.cpu().numpy(), ids.cpu().numpy())
+    np.testing.assert_array_equal(got.cpu().numpy(), want)
+    assert n_piv == len(piv)
+    assert rounds >= 1 and rounds % 4 == 0
