@@ -50,8 +50,9 @@ L2_PROFILE = os.path.join(ROOT, "profiles", "search_kernel_s5_sift2x200k.md")
 PRUNE_KERNELS = {
     0: ("prune_small_kernel", "prune_small_kernel_sift2x500k.txt", "prune_small_kernel_sift2x200k.md"),
     3: ("prune_walk_kernel", "prune_walk_kernel_sift2x500k.txt", "prune_walk_kernel_sift2x200k.md"),
+    4: ("prune_code_kernel", "prune_code_kernel_sift2x500k.txt", "prune_code_kernel_sift2x200k.md"),
 }
-PRUNE_DEFAULT_VARIANT = 3
+PRUNE_DEFAULT_VARIANT = 4   # integer rows
 L2_METRIC, IP_METRIC = 0, 1
 
 
@@ -581,10 +582,12 @@ def run_ours(args, ws, rank, local):
     s_bytes = s_ms = 0.0
     launches = 0
     n_search_launches = 0
+    # integer rows are read as codes, a byte per component (S6 says whether they were)
+    elt = 1 if stats[-1]["prune_kernel"][0] == 4 else 4
     for st in stats:
         for i, ph in ((0, 1), (1, 4), (2, 5)):
-            s_bytes += (st["search_ndc"][i] * W.dim * 4 + st["search_exp"][i] * W.R * 4 +
-                        st["search_queries"][i] * W.dim * 4)
+            s_bytes += (st["search_ndc"][i] * W.dim * elt + st["search_exp"][i] * W.R * 4 +
+                        st["search_queries"][i] * W.dim * elt)
             s_ms += st["phase_ms"][ph]
         launches += st["launches"]
         # one multi-job launch each for S1, S4 and S5 (every pair of the plan)
@@ -607,12 +610,13 @@ def run_ours(args, ws, rank, local):
                    "algorithmic_bytes_per_launch": s_bytes / n_search_launches,
                    "avg_launch_ms": s_ms / n_search_launches,
                    "l2": search_profile_l2(),
+                   "bytes_per_component": elt,
                    "note": "algorithmic bytes; most are served from L2 (see traffic and l2)"}
     # roofline of the S6 source prune, in the unit of its per-owner gather: the
-    # owner row and its c = R + c_cross raw pool rows, d x 4 bytes each, per
+    # owner row and its c = R + c_cross raw pool rows, d x 4 bytes each (coded: d), per
     # owner (every source vertex), against the measured HBM copy bandwidth
     pool = W.R + (W.L + 1) // 2
-    b_per_owner = (pool + 1) * W.dim * 4
+    b_per_owner = (pool + 1) * W.dim * elt
     owners = sum(st["pivots"] + st["followers"] for st in stats)
     p_ms = sum(st["phase_ms"][6] for st in stats)
     n_p6 = len(stats) * (len(plan_used) if plan_used else 1)

@@ -40,7 +40,8 @@
  *                             filter, 2 (default) alone where they are exact
  *     RNSM_PRUNE_VARIANT=v    force prune variant v where it applies (0 the
  *                             FP32 triangle, 1 the pair tile, 2 the general
- *                             tile, 3 the FP32 walk)
+ *                             tile, 3 the FP32 walk, 4 the walk over exact
+ *                             coded rows)
  *     RNSM_TUNE_LOG=1|2       print the prune tuner's choices (2: and slices)
  *                             to stderr
  *     RNSM_SEARCH_PER_JOB=1   run a plan's multi-job searches as one launch
@@ -178,8 +179,9 @@ typedef struct {
     /* The prune kernel that served the last S6 call and the last S7 pool prune
      * (the autotuner's choice): 0 the FP32 register-blocked triangle, 1 the
      * pair tensor-core tile, 2 the general tensor-core tile, 3 the FP32 walk
-     * over kept rows; -1 none ran, or the call replayed a captured CUDA graph
-     * (RNSM_FLAG_GRAPH), whose kernels were chosen when it was captured. */
+     * over kept rows, 4 the walk over exact coded rows; -1 none ran, or the
+     * call replayed a captured CUDA graph (RNSM_FLAG_GRAPH), whose kernels were
+     * chosen when it was captured. */
     int32_t prune_kernel[2];
 } rnsm_stats;
 

@@ -183,34 +183,46 @@ rnsm_status pair_exactness(const SegTable &tab, int32_t dim, int32_t prec, int32
 
 constexpr int kWorkSlots = 16;
 
+// The small state lies together (CtlBlock), so that one clear starts a call and
+// one copy reads the error word and the row statistics.
+struct CtlBlock {
+    int32_t err;
+    CodeStats code_stats;
+    unsigned long long ovf_count, ecount, rechecks, tile_tests;
+    unsigned long long stats[8];
+    unsigned int tile_err[4];
+    int32_t scratch_i[4];
+    int32_t work[kWorkSlots];
+    CodeParams code_params;
+};
+
 void take_ctl(Bump &b, Ctl &c, int64_t max_owners = 0) {
-    c.err = b.take<int32_t>(1);
+    CtlBlock *k = b.take<CtlBlock>(1);
+    c.err = &k->err;
+    c.ovf_count = &k->ovf_count;
+    c.work = k->work;
+    c.stats = k->stats;
+    c.ecount = &k->ecount;
+    c.rechecks = &k->rechecks;
+    c.tile_tests = &k->tile_tests;
+    c.tile_err = k->tile_err;
+    c.scratch_i = k->scratch_i;
+    c.code_stats = &k->code_stats;
+    c.code_params = &k->code_params;
     c.ovf = max_owners > 0 ? b.take<int32_t>(max_owners) : nullptr;
-    c.ovf_count = b.take<unsigned long long>(1);
-    c.work = b.take<int32_t>(kWorkSlots);
-    c.stats = b.take<unsigned long long>(8);
-    c.ecount = b.take<unsigned long long>(1);
-    c.rechecks = b.take<unsigned long long>(1);
-    c.tile_tests = b.take<unsigned long long>(1);
-    c.tile_err = b.take<unsigned int>(4);
-    c.scratch_i = b.take<int32_t>(4);
-    c.code_stats = b.take<CodeStats>(1);
-    c.code_params = b.take<CodeParams>(1);
 }
 
 rnsm_status ctl_reset(const Ctl &c, cudaStream_t st) {
-    CK(cudaMemsetAsync(c.err, 0, sizeof(int32_t), st));
-    CK(cudaMemsetAsync(c.stats, 0, 8 * sizeof(unsigned long long), st));
-    CK(cudaMemsetAsync(c.rechecks, 0, sizeof(unsigned long long), st));
-    CK(cudaMemsetAsync(c.tile_tests, 0, sizeof(unsigned long long), st));
-    CK(cudaMemsetAsync(c.tile_err, 0, 4 * sizeof(unsigned int), st));
+    CK(cudaMemsetAsync(c.err, 0, sizeof(CtlBlock), st));
     return RNSM_OK;
 }
 
-rnsm_status check_err_word(const Ctl &c, cudaStream_t st) {
-    int32_t err = 0;
-    CK(cudaMemcpyAsync(&err, c.err, sizeof(err), cudaMemcpyDeviceToHost, st));
+rnsm_status check_err_word(const Ctl &c, cudaStream_t st, CodeStats *rows = nullptr) {
+    CtlBlock head;
+    CK(cudaMemcpyAsync(&head, c.err, offsetof(CtlBlock, ovf_count), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    const int32_t err = head.err;
+    if (rows) *rows = head.code_stats;
     if (err & 1) return fail(RNSM_EGRAPH, "adjacency holds a vertex id outside [-1, n)");
     if (err & 2) return fail(RNSM_EGRAPH, "vectors hold a non-finite value");
     if (err & 16) return fail(RNSM_EGRAPH, "a prune pool exceeded 4096 candidates");
@@ -276,13 +288,6 @@ rnsm_status check_segments(const rnsm_segment *segs, int32_t m, int32_t R) {
     return RNSM_OK;
 }
 
-rnsm_status validate_on_device(const float *v, int64_t n, int32_t dim, const int32_t *adj,
-                               int32_t r_in, const Ctl &c, cudaStream_t st) {
-    CK(launch_validate_vecs(v, n * dim, c.err, st));
-    if (adj && r_in > 0) CK(launch_validate_graph(adj, n, r_in, c.err, st));
-    return RNSM_OK;
-}
-
 // ------------------------------------------------------------- coded rows
 //
 // A byte per dimension of every row of the call, in a grow-only buffer of its
@@ -324,8 +329,7 @@ uint8_t *codes_acquire(size_t bytes, cudaStream_t st) {
 
 // Validates the rows of the table's first `checked` segments (the error word is
 // read by the caller's check) and, where it pays, codes all of them; *params is
-// valid after that check.  evals: distances that the call's searches are
-// expected to compute.  A row's code costs what some 8 evaluations gain (a pass
+// valid after that check.  evals: distances that the call is expected to compute.  A row's code costs what some 8 evaluations gain (a pass
 // over 5 bytes a dimension against 3 gathered bytes and most of the arithmetic).
 rnsm_status code_table(const SegTable &t, int32_t dim, int32_t metric, int32_t checked, int64_t evals,
                        const Ctl &c, cudaStream_t st, Codes &cd, CodeParams *params) {
@@ -351,6 +355,28 @@ void code_mode(Codes &cd, const CodeParams &p, int32_t dim, int32_t metric) {
     if (p.exact && metric == RNSM_METRIC_L2 && dim <= 256 && codes_allowed() > 1) cd.mode = kCodeExact;
     else if (p.useful) cd.mode = kCodeFilter;
 }
+
+// For calls that only prune: the scan in place of the finite check, and after
+// that check codes only where they are the rows.
+rnsm_status scan_table(const SegTable &t, int32_t dim, int32_t metric, int64_t evals, const Ctl &c, cudaStream_t st,
+                       bool &scanned) {
+    scanned = prune_code_ok(dim, metric) && codes_allowed() > 1 && evals >= 8 * t.off[t.m];
+    if (scanned) CK(launch_code_scan(t, dim, t.m, c.code_stats, c.err, st));
+    return RNSM_OK;
+}
+
+rnsm_status code_scanned(const SegTable &t, int32_t dim, int32_t metric, bool scanned, const CodeStats &rows,
+                         const Ctl &c, cudaStream_t st, const uint8_t **codes) {
+    *codes = nullptr;
+    if (!scanned || !codes_exact(rows)) return RNSM_OK;
+    uint8_t *p = codes_acquire((size_t)t.off[t.m] * dim, st);
+    if (p) CK(launch_code_rows(t, dim, metric, p, c.code_stats, nullptr, st));
+    *codes = p;
+    return RNSM_OK;
+}
+
+// The codes for the prunes: where they are the rows.
+const uint8_t *exact_codes(const Codes &cd) { return cd.mode == kCodeExact ? cd.rows : nullptr; }
 
 // A beam search evaluates some 16 vertices per entry of its beam.
 int64_t search_evals(int64_t queries, int32_t ef) { return 16 * queries * ef; }
@@ -436,7 +462,7 @@ rnsm_status reverse_into(const SegTable &tab, int32_t dim, const rnsm_params &p,
                          const int32_t *eu, const int32_t *ev, int64_t cap,
                          const unsigned long long *count, int32_t key_lo, int64_t nkeys,
                          int32_t csr_max_bound, const RevBufs &r, const Ctl &c, cudaStream_t st,
-                         const QuantBufs *qb = nullptr) {
+                         const QuantBufs *qb = nullptr, const uint8_t *codes = nullptr) {
     CK(launch_bucket(eu, ev, cap, count, nkeys, key_lo, r.offs, r.cursor, r.ids, r.scan_tmp,
                      r.scan_bytes, st));
     int32_t csr_max = csr_max_bound;
@@ -461,6 +487,7 @@ rnsm_status reverse_into(const SegTable &tab, int32_t dim, const rnsm_params &p,
     a.csr_ids = r.ids;
     a.csr_max = csr_max;
     a.out = lists;
+    a.codes = codes;
     a.err = c.err;
     apply_quant(a, qb, c.rechecks, c.tile_err, c.tile_tests);
     return run_prune(a, c.work + 6, c, st, 1);
@@ -597,11 +624,15 @@ rnsm_status rnsm_search(const float *vecs, int64_t n, int32_t dim, const int32_t
     tab.m = 2;
     Codes codes;
     CodeParams code_params;
-    TRY(code_table(tab, dim, metric, 1, nq > kLatencyQueries ? search_evals(nq, ef) : 0, c, st, codes, &code_params));
-    if (adj && r_in > 0) CK(launch_validate_graph(adj, n, r_in, c.err, st));
-    CK(launch_validate_ids(seeds, nq * n_seeds, n, 1, c.err, st));  // -1 or a vertex
-    TRY(check_err_word(c, st));
-    code_mode(codes, code_params, dim, metric);
+    const bool gated = nq <= kLatencyQueries;   // few queries: one wait, at the end
+    if (!gated) TRY(code_table(tab, dim, metric, 1, search_evals(nq, ef), c, st, codes, &code_params));
+    // adjacency and seeds: -1 or a vertex
+    CK(launch_validate(gated ? vecs : nullptr, n * dim, {adj, adj ? n * r_in : 0, n, -1}, {seeds, nq * n_seeds, n, -1},
+                       {}, c.err, st));
+    if (!gated) {
+        TRY(check_err_word(c, st));
+        code_mode(codes, code_params, dim, metric);
+    }
     SearchArgs a = search_defaults();
     a.code_mode = codes.mode;
     a.code_params = c.code_params;
@@ -626,6 +657,7 @@ rnsm_status rnsm_search(const float *vecs, int64_t n, int32_t dim, const int32_t
     a.out_d = out_dists;
     a.out_ndc = out_ndc;
     a.stats = c.stats;
+    a.gate = gated ? c.err : nullptr;
     TRY(run_search(a, c.work, st));
     TRY(check_err_word(c, st));
     return RNSM_OK;
@@ -731,10 +763,13 @@ rnsm_status rnsm_prune(const float *vecs, int64_t n, int32_t dim, const int32_t 
     take_ctl(b, c, nv);
     take_quant(b, n, dim, qprec, metric, qb);
     TRY(ctl_reset(c, st));
-    TRY(validate_on_device(vecs, n, dim, nullptr, 0, c, st));
-    CK(launch_validate_ids(owners, nv, n, 0, c.err, st));
-    if (w_len > 0) CK(launch_validate_ids(pool, nv * w_len, n, 1, c.err, st));
-    TRY(check_err_word(c, st));
+    bool scanned = false;
+    TRY(scan_table(one_table(vecs, n), dim, metric,
+                   prec == RNSM_PREC_FP32 && w_len <= kPruneSmallMax ? nv * w_len : 0, c, st, scanned));
+    CK(launch_validate(scanned ? nullptr : vecs, n * dim, {owners, nv, n, 0}, {pool, nv * w_len, n, -1}, {}, c.err, st));
+    CodeStats rows;
+    const bool gated = qprec == 0 && !scanned && nv <= kGateOwners;   // FP32 kernels: one wait, at the end
+    if (!gated) TRY(check_err_word(c, st, &rows));
     SegTable tab;
     std::memset(&tab, 0, sizeof(tab));
     tab.base[0] = vecs;
@@ -756,9 +791,11 @@ rnsm_status rnsm_prune(const float *vecs, int64_t n, int32_t dim, const int32_t 
     a.out = out;
     a.out_by_index = 1;
     a.err = c.err;
+    TRY(code_scanned(tab, dim, metric, scanned, rows, c, st, &a.codes));
     if (qb.q) CK(launch_quantize(tab, n, dim, qprec, qb.q, qb.qlo, qb.scale, qb.err, qb.norm, st));
     TRY(pair_exactness(tab, dim, qprec, metric, c, st, qb));
     apply_quant(a, &qb, c.rechecks, nullptr, c.tile_tests);
+    a.gate = gated ? c.err : nullptr;
     TRY(run_prune(a, c.work + 8, c, st));
     TRY(check_err_word(c, st));
     return RNSM_OK;
@@ -784,10 +821,12 @@ rnsm_status rnsm_reverse_edges(const float *vecs, int64_t n, int32_t dim, int32_
     take_ctl(b, c, n);
     take_rev(b, n, ne, r);
     TRY(ctl_reset(c, st));
-    TRY(validate_on_device(vecs, n, dim, lists, R, c, st));
-    CK(launch_validate_ids(eu, ne, n, 0, c.err, st));
-    CK(launch_validate_ids(ev, ne, n, 0, c.err, st));
-    TRY(check_err_word(c, st));
+    bool scanned = false;
+    TRY(scan_table(one_table(vecs, n), dim, metric, 16 * ne, c, st, scanned));
+    CK(launch_validate(scanned ? nullptr : vecs, n * dim, {lists, n * R, n, -1}, {eu, ne, n, 0}, {ev, ne, n, 0}, c.err,
+                       st));
+    CodeStats rows;
+    TRY(check_err_word(c, st, &rows));
     SegTable tab;
     std::memset(&tab, 0, sizeof(tab));
     tab.base[0] = vecs;
@@ -798,7 +837,9 @@ rnsm_status rnsm_reverse_edges(const float *vecs, int64_t n, int32_t dim, int32_
     p.R = R;
     p.alpha = alpha;
     p.metric = metric;
-    TRY(reverse_into(tab, dim, p, lists, eu, ev, ne, nullptr, 0, n, -1, r, c, st));
+    const uint8_t *codes = nullptr;
+    TRY(code_scanned(tab, dim, metric, scanned, rows, c, st, &codes));
+    TRY(reverse_into(tab, dim, p, lists, eu, ev, ne, nullptr, 0, n, -1, r, c, st, nullptr, codes));
     TRY(check_err_word(c, st));
     return RNSM_OK;
 }
@@ -916,9 +957,10 @@ rnsm_status rnsm_build_segment(const float *vecs, int64_t n, int32_t dim, const 
         q.ev = ev;
         q.ecount = c.ecount;
         q.err = c.err;
+        q.codes = exact_codes(codes);
         TRY(run_prune(q, c.work + 8, c, st));
         TRY(reverse_into(tab, dim, p, out_adj, eu, ev, bsz * p.R, c.ecount, 0, n, (int32_t)bsz, r,
-                         c, st));
+                         c, st, nullptr, exact_codes(codes)));
         inserted += bsz;
     }
     TRY(check_err_word(c, st));
@@ -1477,6 +1519,7 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
                 q.out = out_adj;
                 q.err = c.err;
                 apply_quant(q, &mb.qb, c.rechecks, c.tile_err, c.tile_tests);
+                q.codes = exact_codes(codes);
                 TRY(run_prune(q, c.work + 8, c, es, 0));
             }
             tm.end(span);
@@ -1484,7 +1527,7 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
             CK(cudaMemsetAsync(c.ecount, 0, sizeof(unsigned long long), es));
             CK(launch_emit_cross(out_adj, p.R, tab, mk, mb.eu, mb.ev, c.ecount, es));
             TRY(reverse_into(tab, dim, p, out_adj, mb.eu, mb.ev, tab.off[m] * p.R, c.ecount, 0,
-                             tab.off[m], -1, mb.rev, c, es, &mb.qb));
+                             tab.off[m], -1, mb.rev, c, es, &mb.qb, exact_codes(codes)));
             CK(cudaMemsetAsync(mb.rev_counts + g0, 0, sizeof(unsigned long long) * (g1 - g0), es));
             CK(cudaMemcpyAsync(mb.rev_counts + g0, c.ecount, sizeof(unsigned long long),
                                cudaMemcpyDeviceToDevice, es));
@@ -1519,11 +1562,13 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
             q.ecount = c.ecount;
             q.err = c.err;
             apply_quant(q, &mb.qb, c.rechecks, c.tile_err, c.tile_tests);
+            q.codes = exact_codes(codes);
             TRY(run_prune(q, c.work + 8, c, es, 0));
             tm.end(span);
             span = graph ? -1 : tm.begin(7);
             TRY(reverse_into(tab, dim, p, out_adj, mb.eu, mb.ev, ns * p.R, c.ecount, t0, nt,
-                             graph ? kReversePoolBound - p.R : -1, mb.rev, c, es, &mb.qb));
+                             graph ? kReversePoolBound - p.R : -1, mb.rev, c, es, &mb.qb,
+                             exact_codes(codes)));
             CK(cudaMemcpyAsync(mb.rev_counts + e, c.ecount, sizeof(unsigned long long),
                                cudaMemcpyDeviceToDevice, es));
             tm.end(span);

@@ -205,6 +205,46 @@ __global__ void validate_vecs_kernel(const float *v, int64_t count, int32_t *err
     }
 }
 
+// Four loads in flight a thread: the checks are passes over memory.
+__device__ __forceinline__ void check_ids(const IdCheck &k, int64_t t, int64_t threads, bool &bad) {
+    int64_t i = t;
+    for (; i + 3 * threads < k.count; i += 4 * threads) {
+        int32_t v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = __ldg(k.ids + i + u * threads);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) bad = bad || v[u] < k.lo || v[u] >= k.bound;
+    }
+    for (; i < k.count; i += threads) {
+        const int32_t v = __ldg(k.ids + i);
+        bad = bad || v < k.lo || v >= k.bound;
+    }
+}
+
+__global__ void __launch_bounds__(256) validate_kernel(const float4 *v, int64_t count4, const IdCheck a, const IdCheck b,
+                                                       const IdCheck c, int32_t *err) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, threads = (int64_t)gridDim.x * blockDim.x;
+    bool bad = false, inf = false;
+    int64_t i = t;
+    for (; i + 3 * threads < count4; i += 4 * threads) {
+        float4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = __ldg(v + i + u * threads);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            inf = inf || !isfinite(x[u].x) || !isfinite(x[u].y) || !isfinite(x[u].z) || !isfinite(x[u].w);
+    }
+    for (; i < count4; i += threads) {
+        const float4 x = __ldg(v + i);
+        inf = inf || !isfinite(x.x) || !isfinite(x.y) || !isfinite(x.z) || !isfinite(x.w);
+    }
+    check_ids(a, t, threads, bad);
+    check_ids(b, t, threads, bad);
+    check_ids(c, t, threads, bad);
+    if (bad) atomicOr(err, 1);
+    if (inf) atomicOr(err, 2);
+}
+
 __global__ void init_lists_kernel(const int32_t *adj, int64_t n, int32_t r_in, int32_t offset,
                                   int32_t *out, int32_t R) {
     const int64_t total = n * R;
@@ -379,6 +419,19 @@ cudaError_t launch_validate_ids(const int32_t *ids, int64_t count, int64_t bound
 cudaError_t launch_validate_vecs(const float *v, int64_t count, int32_t *err, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
     validate_vecs_kernel<<<grid_for(count, 256), 256, 0, st>>>(v, count, err);
+    note_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_validate(const float *v, int64_t count, const IdCheck &a, const IdCheck &b, const IdCheck &c,
+                            int32_t *err, cudaStream_t st) {
+    const int64_t count4 = v ? count / 4 : 0;
+    int64_t most = count4;
+    for (const IdCheck *k : {&a, &b, &c}) most = k->count > most ? k->count : most;
+    if (most <= 0) return cudaSuccess;
+    int64_t g = (most + 1023) / 1024;
+    if (g > 152 * 8) g = 152 * 8;
+    validate_kernel<<<(unsigned)g, 256, 0, st>>>(reinterpret_cast<const float4 *>(v), count4, a, b, c, err);
     note_launches(1);
     return cudaGetLastError();
 }

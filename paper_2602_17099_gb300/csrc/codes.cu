@@ -12,6 +12,8 @@
 // Rows of integers that span at most 255 (SIFT) have s = 1 and e = 0: S is the
 // squared distance itself, and no FP32 row is needed (kCodeExact).
 #include <float.h>
+#include <math.h>
+#include <string.h>
 
 #include "internal.h"
 
@@ -25,14 +27,6 @@ __device__ __forceinline__ uint32_t order_key(float f) {
 }
 __device__ __forceinline__ float order_value(uint32_t u) {
     return __uint_as_float((u & 0x80000000u) ? u ^ 0x80000000u : ~u);
-}
-
-__global__ void code_reset_kernel(CodeStats *s) {
-    s->omin = 0xffffffffu;
-    s->omax = 0u;
-    s->fraction = 0;
-    s->err2 = 0u;
-    s->norm2 = 0u;
 }
 
 // Block-wide reductions of the passes below: one atomic per block and value
@@ -74,7 +68,7 @@ __global__ void __launch_bounds__(256) code_scan_kernel(const SegTable t, int di
     bad = __syncthreads_or(bad);
     if (threadIdx.x == 0) {
         if (lo <= hi) {
-            atomicMin(&s->omin, order_key(lo));
+            atomicMax(&s->omin_inv, ~order_key(lo));
             atomicMax(&s->omax, order_key(hi));
         }
         if (frac) atomicOr(&s->fraction, 1);
@@ -85,7 +79,7 @@ __global__ void __launch_bounds__(256) code_scan_kernel(const SegTable t, int di
 // lo and s of the scanned rows; s = 0: no codes (a range that is empty, not
 // finite, or so large or small that the bounds below could leave FP32's range).
 __device__ __forceinline__ void code_grid(const CodeStats *st, float &lo, float &s) {
-    const float a = order_value(st->omin), b = order_value(st->omax);
+    const float a = order_value(~st->omin_inv), b = order_value(st->omax);
     const float range = b - a;
     lo = a;
     s = 0.f;
@@ -187,8 +181,8 @@ __global__ void __launch_bounds__(1024) code_final_kernel(const SegTable t, int 
     code_grid(st, lo, s);
     p->scale = s;
     p->inv_scale = s > 0.f ? 1.f / s : 0.f;
-    p->exact = s == 1.f && !st->fraction && st->err2 == 0u;
-    const float range = order_value(st->omax) - order_value(st->omin);
+    p->exact = s == 1.f && !st->fraction;
+    const float range = order_value(st->omax) - order_value(~st->omin_inv);
     const float e = 1.001f * sqrtf(__uint_as_float(st->err2)) + 1.2e-7f * sqrtf((float)dim) * range;
     p->err = p->exact ? 0.f : 2.f * e;
     p->norm2 = 1.0001f * __uint_as_float(st->norm2);
@@ -198,15 +192,26 @@ __global__ void __launch_bounds__(1024) code_final_kernel(const SegTable t, int 
 
 }  // namespace
 
+// Whether the scanned rows are their codes (code_grid's s = 1).
+bool codes_exact(const CodeStats &s) {
+    auto value = [](uint32_t u) {
+        const uint32_t b = (u & 0x80000000u) ? u ^ 0x80000000u : ~u;
+        float f;
+        memcpy(&f, &b, sizeof(f));
+        return f;
+    };
+    const float a = value(~s.omin_inv), b = value(s.omax);
+    return !s.fraction && b - a <= 255.f && fabsf(a) <= 65536.f;
+}
+
 bool codes_dim_ok(int dim) { return dim == 64 || dim == 96 || dim == 128 || dim == 256 || dim == 768; }
 
 cudaError_t launch_code_scan(const SegTable &t, int32_t dim, int32_t checked, CodeStats *s, int32_t *err,
                              cudaStream_t st) {
-    code_reset_kernel<<<1, 1, 0, st>>>(s);
     int64_t g = (t.off[t.m] * (dim / 4) + 1023) / 1024;
     if (g > 152 * 8) g = 152 * 8;
     code_scan_kernel<<<(unsigned)(g < 1 ? 1 : g), 256, 0, st>>>(t, dim, checked, s, err);
-    note_launches(2);
+    note_launches(1);
     return cudaGetLastError();
 }
 
@@ -215,8 +220,10 @@ cudaError_t launch_code_rows(const SegTable &t, int32_t dim, int32_t metric, uin
     int64_t g = (t.off[t.m] + 7) / 8;
     if (g > 152 * 8) g = 152 * 8;
     code_rows_kernel<<<(unsigned)(g < 1 ? 1 : g), 256, 0, st>>>(t, dim, codes, s);
+    note_launches(1);
+    if (!p) return cudaGetLastError();
     code_final_kernel<<<1, 1024, 0, st>>>(t, dim, metric, s, p);
-    note_launches(2);
+    note_launches(1);
     return cudaGetLastError();
 }
 

@@ -39,10 +39,10 @@ void note_launches(int n);
 long long launches_so_far();
 
 // Coded rows (codes.cu): a byte per dimension on one grid lo + s * c for all
-// the rows of a call.  CodeStats: what the passes over the rows gather.
+// the rows of a call.  CodeStats: what the passes over the rows gather (starts as zeros).
 // CodeParams: the searches' constants, read on the device.
 struct CodeStats {
-    uint32_t omin, omax;   // smallest and largest component, order-preserving bits
+    uint32_t omin_inv, omax;   // smallest (inverted) and largest component, order-preserving bits
     int32_t fraction;      // a component is no integer
     uint32_t err2, norm2;  // largest squared residual and squared row norm (float bits)
 };
@@ -59,8 +59,10 @@ bool codes_dim_ok(int dim);
 // the statistics, in one pass over the table's rows; then the codes (rows by global id) and the constants.
 cudaError_t launch_code_scan(const SegTable &t, int32_t dim, int32_t checked, CodeStats *s, int32_t *err,
                              cudaStream_t st);
+// (p null: no constants.)
 cudaError_t launch_code_rows(const SegTable &t, int32_t dim, int32_t metric, uint8_t *codes, CodeStats *s,
                              CodeParams *p, cudaStream_t st);
+bool codes_exact(const CodeStats &s);
 // Launches of up to this many queries take the search's latency shape, which
 // does not filter by codes.
 constexpr int64_t kLatencyQueries = 1216;
@@ -121,6 +123,7 @@ struct SearchArgs {
     int64_t *out_ndc;         // nullable, [nq]
     unsigned long long *stats;  // nullable: [0] += NDC, [1] += expansions
     int32_t *work;            // zeroed work counter
+    const int32_t *gate;      // nullable: an error word of the input checks; set bits 1 or 2: no work
     int32_t code_mode;        // CodeMode of the launch
     const uint8_t *codes;     // coded rows of base and of qvecs
     const uint8_t *qcodes;
@@ -183,15 +186,18 @@ struct PruneArgs {
     unsigned int *tile_err;   // nullable [4]: sampled tile error maxima (float bits) and count
     int32_t *work;
     int32_t *work2;           // second zeroed counter (overflow pass)
+    const int32_t *gate;      // nullable, FP32 kernels: as SearchArgs::gate
     int32_t *ovf_list;        // [n_owners]: owners whose pool exceeds the small-pool kernel
     unsigned long long *ovf_count;
     int32_t *err;             // bit 4: pool larger than the capacity; bit 6: tile wait ran out
     int32_t test_withhold_commit;  // test-only (tensor-core prune): never signal MMA completion
+    const uint8_t *codes;     // nullable: exact coded rows by global id (codes.cu)
     int32_t pair_hi_only;     // pair tile: integer rows spanning <= 256, hi terms only
 };
 
 // variant (optional): set to the prune variant that served the call (0 the
-// FP32 triangle, 1 the pair tile, 2 the general tile, 3 the FP32 walk).
+// FP32 triangle, 1 the pair tile, 2 the general tile, 3 the FP32 walk, 4 the walk
+// over exact coded rows).
 cudaError_t launch_prune(const PruneArgs &a, cudaStream_t st, int *variant = nullptr);
 // The FP32 kernels behind it: the small-pool kernel (raw pools of at most
 // kPruneSmallMax; larger ones go to a->ovf_list) and the general kernel (with
@@ -201,6 +207,9 @@ cudaError_t launch_small(const PruneArgs &a, cudaStream_t st);
 // The same pools (d <= kPruneWalkMaxDim) by the walk over kept rows only.
 constexpr int kPruneWalkMaxDim = 128;
 cudaError_t launch_walk(const PruneArgs &a, cudaStream_t st);
+// The same pools where the rows are exact codes (a.codes; L2, d = 64, 96, 128).
+bool prune_code_ok(int dim, int metric);
+cudaError_t launch_prune_code(const PruneArgs &a, cudaStream_t st);
 cudaError_t launch_prune_general(const PruneArgs &a, const int32_t *idx_list,
                                  const unsigned long long *idx_count, cudaStream_t st);
 
@@ -307,6 +316,18 @@ cudaError_t launch_validate_graph(const int32_t *adj, int64_t n, int32_t r_in, i
 cudaError_t launch_validate_ids(const int32_t *ids, int64_t count, int64_t bound,
                                 int32_t allow_minus1, int32_t *err, cudaStream_t st);
 cudaError_t launch_validate_vecs(const float *v, int64_t count, int32_t *err, cudaStream_t st);
+// Several checks in one launch: count floats of v finite (bit 2 of *err; v null:
+// none), every id list within [lo, bound) (bit 1).
+struct IdCheck {
+    const int32_t *ids = nullptr;
+    int64_t count = 0, bound = 0;
+    int32_t lo = 0;
+};
+cudaError_t launch_validate(const float *v, int64_t count, const IdCheck &a, const IdCheck &b, const IdCheck &c,
+                            int32_t *err, cudaStream_t st);
+// Calls of up to this many owners leave the check of their inputs to the kernels
+// (SearchArgs::gate, PruneArgs::gate) instead of waiting for it on the host.
+constexpr int64_t kGateOwners = 65536;
 cudaError_t launch_init_lists(const int32_t *adj, int64_t n, int32_t r_in, int32_t offset,
                               int32_t *out, int32_t R, cudaStream_t st);
 cudaError_t launch_fill(int32_t *p, int64_t count, int32_t value, cudaStream_t st);

@@ -92,16 +92,21 @@ extern "C" rnsm_status rnsm_prune_noalloc(const float *vecs, int64_t n, int32_t 
     // the array keeps the previous call's contents: zero the counters and the error word
     e = cudaMemsetAsync(base, 0, kHeadBytes, st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
-    if ((e = rnsm::launch_validate_vecs(vecs, n * dim, err, st)) != cudaSuccess ||
-        (e = rnsm::launch_validate_ids(owners, nv, n, 0, err, st)) != cudaSuccess ||
-        (w_len > 0 && (e = rnsm::launch_validate_ids(pool, nv * w_len, n, 1, err, st)) != cudaSuccess))
+    if ((e = rnsm::launch_validate(vecs, n * dim, {owners, nv, n, 0}, {pool, nv * w_len, n, -1}, {}, err, st)) !=
+        cudaSuccess)
         return cuda_fail(e, "validation launch");
     int32_t herr = 0;
-    if ((e = cudaMemcpyAsync(&herr, err, sizeof(herr), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(st)) != cudaSuccess)
+    // small calls: the prune kernels look at the error word themselves, and the host
+    // waits once (a second wait is a quarter of a call of 75 owners)
+    const bool gated = nv <= rnsm::kGateOwners;
+    if (!gated && ((e = cudaMemcpyAsync(&herr, err, sizeof(herr), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
+                   (e = cudaStreamSynchronize(st)) != cudaSuccess))
         return cuda_fail(e, "validation read-back");
-    if (herr & 1) return fail(RNSM_EGRAPH, "an owner or pool id is outside its range");
-    if (herr & 2) return fail(RNSM_EGRAPH, "vectors hold a non-finite value");
+    auto invalid = [&] {
+        return herr & 1 ? fail(RNSM_EGRAPH, "an owner or pool id is outside its range")
+                        : fail(RNSM_EGRAPH, "vectors hold a non-finite value");
+    };
+    if (herr & 3) return invalid();
 
     rnsm::PruneArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -125,10 +130,12 @@ extern "C" rnsm_status rnsm_prune_noalloc(const float *vecs, int64_t n, int32_t 
     a.ovf_list = ovf_list;
     a.ovf_count = ovf_count;
     a.err = err;
+    a.gate = gated ? err : nullptr;
     if ((e = rnsm::launch_prune(a, st)) != cudaSuccess) return cuda_fail(e, "prune launch");
     if ((e = cudaMemcpyAsync(&herr, err, sizeof(herr), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
         (e = cudaStreamSynchronize(st)) != cudaSuccess)
         return cuda_fail(e, "prune");
+    if (herr & 3) return invalid();
     if (herr & 16) return fail(RNSM_EGRAPH, "a prune pool exceeded 4096 candidates");
     if (herr) return fail(RNSM_ECUDA, "device error word set");
     return RNSM_OK;

@@ -165,6 +165,7 @@ __global__ void __launch_bounds__(kThreads) prune_kernel(const PruneArgs a, int 
     const int dim = a.dim;
     const int R = a.R;
     const int metric = a.metric;
+    if (a.gate && (*a.gate & 3)) return;   // the inputs did not pass their checks
 
     // owners: all of [0, n_owners), or the listed ones (pools the small-pool kernel passed on)
     const int64_t n_items = idx_list ? (int64_t)*idx_count : a.n_owners;
@@ -530,6 +531,7 @@ __global__ void __launch_bounds__(kSmallThreads, RNSM_SMALL_MIN_BLOCKS) prune_sm
     const int dim = a.dim;
     const int R = a.R;
     const int metric = a.metric;
+    if (a.gate && (*a.gate & 3)) return;   // the inputs did not pass their checks
     for (;;) {
         if (tid == 0) sh_i = atomicAdd(a.work, chunk);
         __syncthreads();
@@ -848,6 +850,7 @@ __global__ void __launch_bounds__(kWalkThreads, walk_min_blocks<kF4>())
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int dim = a.dim, F4 = dim >> 2;
     const int R = a.R;
+    if (a.gate && (*a.gate & 3)) return;   // the inputs did not pass their checks
     // this thread's candidate row; the next owner's is loaded into it at the end
     // of an owner's walk, so its latency overlaps the output and the claim
     float4 xr[kWalkMaxF4];

@@ -1,0 +1,299 @@
+// The occlusion prune over coded rows (codes.cu) where the codes are the rows:
+// integers spanning up to 255 (SIFT), L2, pools of at most 64 raw candidates.
+// Every distance is then an exact integer below 2^24, the same that the FP32
+// chain gives, and the decisions are the FP32 ones.
+//
+// What bounds the FP32 walk (prune.cu) is that a row of 128 floats a thread
+// leaves twelve warps per SM, each waiting on shared memory and barriers.  A
+// coded row is 32 words: one warp takes an owner alone, two rows a lane, without
+// any barrier, and a pair costs 32 dp4a (norms are computed once) instead of 128
+// packed FP32 operations.  2 x 500k SIFT-like rows (d = 128): S6 13.3 -> 2.40 ms, S7
+// 9.7 -> 2.43 ms.  Twenty warps per SM; 16 with registers to spare: 2.47 ms.
+//
+// Per owner (one warp): the rows by cp.async into shared memory; every lane its
+// two candidates' distances to the owner; positions by counting (64-bit keys:
+// distance, id, slot); each lane its two positions' rows into registers; then the
+// greedy walk kept row by kept row: the lowest open position is kept, its row is
+// read as a broadcast, and the positions after it that it occludes close.
+#include "internal.h"
+
+namespace rnsm {
+
+namespace {
+
+constexpr int kCodeWarps = 4;
+constexpr int kPool = 64;
+
+template <int W>   // words of a row: 16, 24, 32 (d = 64, 96, 128)
+struct CodePool {
+    static constexpr int kStride = W + 4;   // words; 8 lanes' 16-byte reads fall on 32 banks
+    uint32_t rows[kPool * kStride];
+    uint32_t owner[W];
+    unsigned long long key[kPool];     // raw order
+    unsigned long long order[kPool];   // position order
+    int32_t norm[kPool];
+    int32_t id[kPool];
+};
+
+template <int W>
+constexpr int code_blocks() { return W == 32 ? 5 : W == 24 ? 6 : 8; }
+
+__device__ __forceinline__ void cp_async16(uint32_t *dst, const uint8_t *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+                 "l"(src)
+                 : "memory");
+}
+
+template <int W>
+__global__ void __launch_bounds__(kCodeWarps * 32, code_blocks<W>())
+    prune_code_kernel(const PruneArgs a, int chunk) {
+    constexpr int kStride = CodePool<W>::kStride, kVec = W / 4;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    CodePool<W> &s = reinterpret_cast<CodePool<W> *>(smem_raw)[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const int R = a.R;
+    for (;;) {
+        int32_t claim = 0;
+        if (lane == 0) claim = atomicAdd(a.work, chunk);
+        const int64_t i0 = __shfl_sync(0xffffffffu, claim, 0);
+        if (i0 >= a.n_owners) break;
+        const int64_t i1 = min(a.n_owners, i0 + chunk);
+        for (int64_t i = i0; i < i1; ++i) {
+            const int32_t owner = a.owner_ids ? a.owner_ids[i] : (int32_t)(a.owner_base + i);
+            int64_t c_lo = 0, c_hi = 0;
+            if (a.csr_offs) {
+                c_lo = a.csr_offs[i];
+                c_hi = a.csr_offs[i + 1];
+            }
+            if (a.skip_empty_csr && c_hi == c_lo) continue;
+            const int64_t nr_raw = (int64_t)a.lenA + a.lenB + (c_hi - c_lo);
+            if (nr_raw > kPool) {
+                if (lane == 0) a.ovf_list[atomicAdd(a.ovf_count, 1ull)] = (int32_t)i;
+                continue;
+            }
+            const int nr = (int)nr_raw;
+            // 1. the pool's ids, and every row (and the owner's) on its way
+            int32_t id[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int j = lane + 32 * h;
+                int32_t c = -1;
+                if (j < nr) {
+                    if (j < a.lenA) {
+                        c = a.listA[(int64_t)owner * a.lenA + j];
+                    } else if (j < a.lenA + a.lenB) {
+                        c = a.listB[i * a.strideB + (j - a.lenA)];
+                        if (c >= 0) c += a.offB;
+                    } else {
+                        c = a.csr_ids[c_lo + (j - a.lenA - a.lenB)];
+                    }
+                    if (c == owner) c = -1;
+                }
+                id[h] = c;
+                s.id[j] = c;
+            }
+            __syncwarp();
+            if (lane < kVec) cp_async16(s.owner + 4 * lane, a.codes + (int64_t)owner * (4 * W) + 16 * lane);
+            for (int c = lane; c < nr * kVec; c += 32) {
+                const int r = c / kVec, f = c - r * kVec;
+                const int32_t g = s.id[r];
+                if (g >= 0) cp_async16(s.rows + r * kStride + 4 * f, a.codes + (int64_t)g * (4 * W) + 16 * f);
+            }
+            asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+            __syncwarp();
+            // 2. keys: distance to the owner, id, slot (none repeats)
+            const bool two = nr > 32;
+            uint32_t nv = 0u, n0 = 0u, n1 = 0u, v0 = 0u, v1 = 0u;
+            const uint4 *r0 = reinterpret_cast<const uint4 *>(s.rows + lane * kStride);
+            const uint4 *r1 = reinterpret_cast<const uint4 *>(s.rows + (lane + 32) * kStride);
+#pragma unroll
+            for (int f = 0; f < kVec; ++f) {
+                const uint4 o = reinterpret_cast<const uint4 *>(s.owner)[f];
+                nv = __dp4a(o.x, o.x, __dp4a(o.y, o.y, __dp4a(o.z, o.z, __dp4a(o.w, o.w, nv))));
+                const uint4 x = r0[f];
+                n0 = __dp4a(x.x, x.x, __dp4a(x.y, x.y, __dp4a(x.z, x.z, __dp4a(x.w, x.w, n0))));
+                v0 = __dp4a(x.x, o.x, __dp4a(x.y, o.y, __dp4a(x.z, o.z, __dp4a(x.w, o.w, v0))));
+                if (two) {
+                    const uint4 y = r1[f];
+                    n1 = __dp4a(y.x, y.x, __dp4a(y.y, y.y, __dp4a(y.z, y.z, __dp4a(y.w, y.w, n1))));
+                    v1 = __dp4a(y.x, o.x, __dp4a(y.y, o.y, __dp4a(y.z, o.z, __dp4a(y.w, o.w, v1))));
+                }
+            }
+            s.norm[lane] = (int32_t)n0;
+            s.norm[lane + 32] = (int32_t)n1;
+            unsigned long long K[2];
+            K[0] = (id[0] >= 0 ? ((unsigned long long)(nv + n0 - 2u * v0) << 37) | ((unsigned long long)(uint32_t)id[0] << 6)
+                               : ~63ull) | (unsigned)lane;
+            K[1] = (id[1] >= 0 ? ((unsigned long long)(nv + n1 - 2u * v1) << 37) | ((unsigned long long)(uint32_t)id[1] << 6)
+                               : ~63ull) | (unsigned)(lane + 32);
+            s.key[lane] = K[0];
+            s.key[lane + 32] = K[1];
+            __syncwarp();
+            // 3. position = number of smaller keys
+            {
+                int p0 = 0, p1 = 0;
+                const ulonglong2 *kk = reinterpret_cast<const ulonglong2 *>(s.key);
+                const int half = two ? 32 : 16;
+#pragma unroll 8
+                for (int k = 0; k < half; ++k) {
+                    const ulonglong2 q = kk[k];
+                    p0 += (q.x < K[0] ? 1 : 0) + (q.y < K[0] ? 1 : 0);
+                    p1 += (q.x < K[1] ? 1 : 0) + (q.y < K[1] ? 1 : 0);
+                }
+                s.order[p0] = K[0];
+                if (two) s.order[p1] = K[1];
+                else s.order[lane + 32] = K[1];
+            }
+            __syncwarp();
+            K[0] = s.order[lane];
+            K[1] = s.order[lane + 32];
+            id[0] = (int32_t)((K[0] >> 6) & 0x7fffffffull);
+            id[1] = (int32_t)((K[1] >> 6) & 0x7fffffffull);
+            // live positions: valid and not a repeat of the previous id
+            const bool ok0 = K[0] < ~63ull, ok1 = K[1] < ~63ull;
+            const int32_t pr0 = lane ? (int32_t)((s.order[lane - 1] >> 6) & 0x7fffffffull) : -1;
+            const int32_t pr1 = (int32_t)((s.order[lane + 31] >> 6) & 0x7fffffffull);
+            const unsigned long long live =
+                (unsigned long long)__ballot_sync(0xffffffffu, ok0 && pr0 != id[0]) |
+                ((unsigned long long)__ballot_sync(0xffffffffu, ok1 && pr1 != id[1]) << 32);
+            unsigned long long kept = 0ull;
+            if (a.keep_all_if_fit && __popcll(live) <= R) {
+                kept = live;
+            } else {
+                // 4. the walk
+                uint32_t x0[W], x1[W];
+                const int s0 = (int)(K[0] & 63ull), s1 = (int)(K[1] & 63ull);
+                const uint4 *q0 = reinterpret_cast<const uint4 *>(s.rows + s0 * kStride);
+                const uint4 *q1 = reinterpret_cast<const uint4 *>(s.rows + s1 * kStride);
+#pragma unroll
+                for (int f = 0; f < kVec; ++f) {
+                    const uint4 x = q0[f];
+                    x0[4 * f] = x.x;
+                    x0[4 * f + 1] = x.y;
+                    x0[4 * f + 2] = x.z;
+                    x0[4 * f + 3] = x.w;
+                    const uint4 y = q1[f];
+                    x1[4 * f] = y.x;
+                    x1[4 * f + 1] = y.y;
+                    x1[4 * f + 2] = y.z;
+                    x1[4 * f + 3] = y.w;
+                }
+                const int32_t m0 = s.norm[s0], m1 = s.norm[s1];
+                const float dv0 = (float)(uint32_t)(K[0] >> 37), dv1 = (float)(uint32_t)(K[1] >> 37);
+                unsigned long long open = live;
+                int nk = 0;
+                while (open && nk < R) {
+                    const int p = __ffsll((long long)open) - 1;
+                    kept |= 1ull << p;
+                    ++nk;
+                    open &= open - 1ull;
+                    if (!open) break;
+                    const int ss = (int)(reinterpret_cast<const uint32_t *>(s.order)[2 * p] & 63u);
+                    const uint4 *row = reinterpret_cast<const uint4 *>(s.rows + ss * kStride);
+                    const int32_t ns = s.norm[ss];
+                    unsigned d0 = 0u, d1 = 0u;
+                    const unsigned o0 = (unsigned)open, o1 = (unsigned)(open >> 32);
+                    // (a half without open positions is left out)
+                    if (o0 && o1) {
+                        uint32_t t0 = 0u, t1 = 0u;
+#pragma unroll
+                        for (int f = 0; f < kVec; ++f) {
+                            const uint4 o = row[f];
+                            t0 = __dp4a(x0[4 * f], o.x, __dp4a(x0[4 * f + 1], o.y, __dp4a(x0[4 * f + 2], o.z, __dp4a(x0[4 * f + 3], o.w, t0))));
+                            t1 = __dp4a(x1[4 * f], o.x, __dp4a(x1[4 * f + 1], o.y, __dp4a(x1[4 * f + 2], o.z, __dp4a(x1[4 * f + 3], o.w, t1))));
+                        }
+                        d0 = __ballot_sync(0xffffffffu, fmaf(a.alpha, (float)(ns + m0 - 2 * (int32_t)t0), -dv0) <= 0.f);
+                        d1 = __ballot_sync(0xffffffffu, fmaf(a.alpha, (float)(ns + m1 - 2 * (int32_t)t1), -dv1) <= 0.f);
+                    } else {
+                        uint32_t t0 = 0u, t1 = 0u;
+                        if (o0) {
+#pragma unroll
+                            for (int f = 0; f < kVec; ++f) {
+                                const uint4 o = row[f];
+                                t0 = __dp4a(x0[4 * f], o.x, __dp4a(x0[4 * f + 1], o.y, t0));
+                                t1 = __dp4a(x0[4 * f + 2], o.z, __dp4a(x0[4 * f + 3], o.w, t1));
+                            }
+                            d0 = __ballot_sync(0xffffffffu, fmaf(a.alpha, (float)(ns + m0 - 2 * (int32_t)(t0 + t1)), -dv0) <= 0.f);
+                        } else {
+#pragma unroll
+                            for (int f = 0; f < kVec; ++f) {
+                                const uint4 o = row[f];
+                                t0 = __dp4a(x1[4 * f], o.x, __dp4a(x1[4 * f + 1], o.y, t0));
+                                t1 = __dp4a(x1[4 * f + 2], o.z, __dp4a(x1[4 * f + 3], o.w, t1));
+                            }
+                            d1 = __ballot_sync(0xffffffffu, fmaf(a.alpha, (float)(ns + m1 - 2 * (int32_t)(t0 + t1)), -dv1) <= 0.f);
+                        }
+                    }
+                    open &= ~((unsigned long long)d0 | ((unsigned long long)d1 << 32));
+                }
+            }
+            // 5. output in (distance, id) order: the kept positions
+            {
+                const int nk = __popcll(kept);
+                int32_t *out = a.out + (a.out_by_index ? i : (int64_t)owner) * R;
+                const bool k0 = (kept >> lane) & 1ull, k1 = (kept >> (lane + 32)) & 1ull;
+                if (k0) out[__popcll(kept & ((1ull << lane) - 1ull))] = id[0];
+                if (k1) out[__popcll(kept & ((1ull << (lane + 32)) - 1ull))] = id[1];
+                for (int j = nk + lane; j < R; j += 32) out[j] = -1;
+                if (a.eu) {
+                    const bool e0 = k0 && id[0] >= a.emit_lo && id[0] < a.emit_hi;
+                    const bool e1 = k1 && id[1] >= a.emit_lo && id[1] < a.emit_hi;
+                    const unsigned b0 = __ballot_sync(0xffffffffu, e0);
+                    const unsigned b1 = __ballot_sync(0xffffffffu, e1);
+                    const int cnt = __popc(b0) + __popc(b1);
+                    int base = 0;
+                    if (lane == 0 && cnt) base = (int)atomicAdd(a.ecount, (unsigned long long)cnt);
+                    base = __shfl_sync(0xffffffffu, base, 0);
+                    if (e0) {
+                        const int slot = base + __popc(b0 & lanemask_lt());
+                        a.eu[slot] = id[0];
+                        a.ev[slot] = owner;
+                    }
+                    if (e1) {
+                        const int slot = base + __popc(b0) + __popc(b1 & lanemask_lt());
+                        a.eu[slot] = id[1];
+                        a.ev[slot] = owner;
+                    }
+                }
+            }
+            __syncwarp();   // the owner's shared state is free
+        }
+    }
+}
+
+template <int W>
+cudaError_t launch_code_t(const PruneArgs &a, cudaStream_t st) {
+    auto kern = prune_code_kernel<W>;
+    constexpr int smem = kCodeWarps * (int)sizeof(CodePool<W>);
+    static GridCache cache;
+    int64_t grid = 0;
+    cudaError_t e = cached_grid(cache, grid, [&](int dev, int &blocks) {
+        cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (r != cudaSuccess) return r;
+        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        int sms = 0, per_sm = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kCodeWarps * 32, smem);
+        blocks = sms * (per_sm < 1 ? 1 : per_sm);
+        return r;
+    });
+    if (e != cudaSuccess) return e;
+    const int chunk = a.skip_empty_csr ? 8 : 2;
+    const int64_t want = (a.n_owners + (int64_t)kCodeWarps * chunk - 1) / ((int64_t)kCodeWarps * chunk);
+    if (want < grid) grid = want;
+    kern<<<(unsigned)grid, kCodeWarps * 32, smem, st>>>(a, chunk);
+    note_launches(1);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+bool prune_code_ok(int dim, int metric) { return metric == 0 && (dim == 64 || dim == 96 || dim == 128); }
+
+cudaError_t launch_prune_code(const PruneArgs &a, cudaStream_t st) {
+    if (!a.codes || !prune_code_ok(a.dim, a.metric)) return cudaErrorInvalidValue;
+    return a.dim == 64 ? launch_code_t<16>(a, st) : a.dim == 96 ? launch_code_t<24>(a, st) : launch_code_t<32>(a, st);
+}
+
+}  // namespace rnsm

@@ -20,8 +20,15 @@ namespace {
 //             at L2 with the FP32 rows split into two terms, or the library's
 //             stored BF16 / E4M3 terms);
 //   kVarFp32: the FP32 kernels (register-blocked triangle for pools <= 64);
-//   kVarWalk: the FP32 walk over kept rows (pools <= 64, d <= 128).
-enum { kVarFp32 = 0, kVarPair = 1, kVarTile = 2, kVarWalk = 3, kVarCount = 4 };
+//   kVarWalk: the FP32 walk over kept rows (pools <= 64, d <= 128);
+//   kVarCode: the walk over exact coded rows (pools <= 64; where the call has them:
+//             integer rows, L2, d = 64, 96, 128).
+enum { kVarFp32 = 0, kVarPair = 1, kVarTile = 2, kVarWalk = 3, kVarCode = 4, kVarCount = 5 };
+
+int forced_prune_variant() {
+    const char *f = getenv("RNSM_PRUNE_VARIANT");
+    return f && f[0] >= '0' && f[0] < '0' + kVarCount ? f[0] - '0' : -1;
+}
 
 // One variant over a call's owners: its kernel for the pools it takes, the
 // general FP32 kernel for the owners whose pools exceed that kernel's capacity.
@@ -41,6 +48,7 @@ cudaError_t run_variant(const PruneArgs &a, int var, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     e = pair ? launch_prune_pair(a, st)
         : tc ? launch_prune_tc(a, st, terms)
+        : var == kVarCode ? launch_prune_code(a, st)
         : var == kVarWalk ? launch_walk(a, st)
         : launch_small(a, st);
     if (e != cudaSuccess) return e;
@@ -56,6 +64,15 @@ cudaError_t run_variant(const PruneArgs &a, int var, cudaStream_t st) {
 // The variants that apply to a call, the default (the first) included.
 int variants_of(const PruneArgs &a, int *out) {
     int n = 0;
+    // exact coded rows: a quarter of the bytes and an eighth of the instructions of
+    // FP32 rows (2 x 500k SIFT-like rows, S6 + S7: 4.8 ms; the FP32 walk 23.0, the
+    // BF16 pair tile 12.5, the FP8 one 14.7), so in FP32 mode nothing else is tried.
+    // With tiles asked for they are one of the tuner's choices, not the default.
+    const bool code_ok = a.codes && prune_code_ok(a.dim, a.metric) && a.lenA + a.lenB <= kPruneSmallMax;
+    if (code_ok && a.prec == 0) {
+        out[n++] = kVarCode;
+        if (forced_prune_variant() < 0) return n;
+    }
     if (a.prec != 0) {
         const bool pair_ok = prune_pair_ok(a.dim, a.prec, a.metric);
         if (pair_ok && a.lenA + a.lenB <= prune_pair_max_pool()) out[n++] = kVarPair;
@@ -65,6 +82,7 @@ int variants_of(const PruneArgs &a, int *out) {
             a.lenA + a.lenB <= prune_tc_max_pool())
             out[n++] = kVarTile;
     }
+    if (code_ok && a.prec != 0) out[n++] = kVarCode;
     // FP32 defaults (calls too small to tune): the walk for the source pools, the
     // triangle for reverse-edge pools (on deep-like rows the walk lost there by 40 %)
     const bool walk_ok = a.dim <= kPruneWalkMaxDim && a.lenA + a.lenB <= kPruneSmallMax;
@@ -118,10 +136,6 @@ struct PruneKey {
 std::mutex g_ptune_mu;
 std::map<PruneKey, int> g_ptuned;
 
-int forced_prune_variant() {
-    const char *f = getenv("RNSM_PRUNE_VARIANT");
-    return f && f[0] >= '0' && f[0] < '0' + kVarCount ? f[0] - '0' : -1;
-}
 
 }  // namespace
 
@@ -134,7 +148,7 @@ cudaError_t launch_prune(const PruneArgs &a, cudaStream_t st, int *variant) {
     const int nv = variants_of(a, vars);
     auto run = [&](const PruneArgs &x, int v) {
         ran = v;
-        if ((v == kVarFp32 || v == kVarWalk) && x.prec != 0) {
+        if ((v == kVarFp32 || v == kVarWalk || v == kVarCode) && x.prec != 0) {
             PruneArgs y = x;
             y.prec = 0;
             return run_variant(y, v, st);

@@ -408,6 +408,7 @@ search_kernel(const SearchArgs a, uint32_t sets, int prefetch) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
+    if (a.gate && (*a.gate & 3)) return;   // the inputs did not pass their checks
     int32_t *tab = reinterpret_cast<int32_t *>(smem + (size_t)warp * warp_smem_bytes(sets, EFMAX, MODE == kCodeFilter ? F4 : 0));
     int32_t *ci = tab + sets * 8;
     int32_t *pass = ci + kBatch;
