@@ -10,7 +10,8 @@
  *   that the library grows on demand and keeps until rnsm_release_workspace()
  *   or process exit.  Calls that search dimensions of 64 and more also keep a
  *   byte per component of their rows (coded rows, kept and released alike; if
- *   there is no memory for them the searches read the FP32 rows alone).
+ *   there is no memory for them the FP32 rows are read alone), and so do the
+ *   larger FP32 prunes of 64, 96 and 128 dimensions.
  * - Vectors are row-major float32, rows contiguous, 16-byte aligned (dim must
  *   be a multiple of 4, at most 1024).  Calls that search (rnsm_search,
  *   rnsm_expand, rnsm_build_segment, rnsm_merge) need a dimension the search
@@ -36,12 +37,13 @@
  *   keep the fastest for the process; every variant gives the same results.
  *   Environment variables read at each call (none changes a result):
  *     RNSM_SEARCH_VARIANT=v   force search launch variant v (0..3)
- *     RNSM_SEARCH_CODES=c     coded rows in the searches: 0 none, 1 only as a
- *                             filter, 2 (default) alone where they are exact
+ *     RNSM_SEARCH_CODES=c     coded rows in searches and FP32 prunes: 0 none,
+ *                             1 only as a filter, 2 (default) alone where they
+ *                             are exact
  *     RNSM_PRUNE_VARIANT=v    force prune variant v where it applies (0 the
  *                             FP32 triangle, 1 the pair tile, 2 the general
- *                             tile, 3 the FP32 walk, 4 the walk over exact
- *                             coded rows)
+ *                             tile, 3 the FP32 walk, 4 the walk over coded
+ *                             rows)
  *     RNSM_TUNE_LOG=1|2       print the prune tuner's choices (2: and slices)
  *                             to stderr
  *     RNSM_SEARCH_PER_JOB=1   run a plan's multi-job searches as one launch
@@ -179,7 +181,7 @@ typedef struct {
     /* The prune kernel that served the last S6 call and the last S7 pool prune
      * (the autotuner's choice): 0 the FP32 register-blocked triangle, 1 the
      * pair tensor-core tile, 2 the general tensor-core tile, 3 the FP32 walk
-     * over kept rows, 4 the walk over exact coded rows; -1 none ran, or the
+     * over kept rows, 4 the walk over coded rows; -1 none ran, or the
      * call replayed a captured CUDA graph (RNSM_FLAG_GRAPH), whose kernels were
      * chosen when it was captured. */
     int32_t prune_kernel[2];

@@ -183,8 +183,7 @@ rnsm_status pair_exactness(const SegTable &tab, int32_t dim, int32_t prec, int32
 
 constexpr int kWorkSlots = 16;
 
-// The small state lies together (CtlBlock), so that one clear starts a call and
-// one copy reads the error word and the row statistics.
+// The small state lies together, so that one clear starts a call.
 struct CtlBlock {
     int32_t err;
     CodeStats code_stats;
@@ -217,12 +216,10 @@ rnsm_status ctl_reset(const Ctl &c, cudaStream_t st) {
     return RNSM_OK;
 }
 
-rnsm_status check_err_word(const Ctl &c, cudaStream_t st, CodeStats *rows = nullptr) {
-    CtlBlock head;
-    CK(cudaMemcpyAsync(&head, c.err, offsetof(CtlBlock, ovf_count), cudaMemcpyDeviceToHost, st));
+rnsm_status check_err_word(const Ctl &c, cudaStream_t st) {
+    int32_t err = 0;
+    CK(cudaMemcpyAsync(&err, c.err, sizeof(err), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    const int32_t err = head.err;
-    if (rows) *rows = head.code_stats;
     if (err & 1) return fail(RNSM_EGRAPH, "adjacency holds a vertex id outside [-1, n)");
     if (err & 2) return fail(RNSM_EGRAPH, "vectors hold a non-finite value");
     if (err & 16) return fail(RNSM_EGRAPH, "a prune pool exceeded 4096 candidates");
@@ -356,27 +353,12 @@ void code_mode(Codes &cd, const CodeParams &p, int32_t dim, int32_t metric) {
     else if (p.useful) cd.mode = kCodeFilter;
 }
 
-// For calls that only prune: the scan in place of the finite check, and after
-// that check codes only where they are the rows.
-rnsm_status scan_table(const SegTable &t, int32_t dim, int32_t metric, int64_t evals, const Ctl &c, cudaStream_t st,
-                       bool &scanned) {
-    scanned = prune_code_ok(dim, metric) && codes_allowed() > 1 && evals >= 8 * t.off[t.m];
-    if (scanned) CK(launch_code_scan(t, dim, t.m, c.code_stats, c.err, st));
-    return RNSM_OK;
+// The codes for the prunes.
+void prune_codes(PruneArgs &a, const Codes &cd, const Ctl &c) {
+    if (cd.mode == kCodeNone) return;
+    a.codes = cd.rows;
+    a.code_params = cd.mode == kCodeExact ? nullptr : c.code_params;
 }
-
-rnsm_status code_scanned(const SegTable &t, int32_t dim, int32_t metric, bool scanned, const CodeStats &rows,
-                         const Ctl &c, cudaStream_t st, const uint8_t **codes) {
-    *codes = nullptr;
-    if (!scanned || !codes_exact(rows)) return RNSM_OK;
-    uint8_t *p = codes_acquire((size_t)t.off[t.m] * dim, st);
-    if (p) CK(launch_code_rows(t, dim, metric, p, c.code_stats, nullptr, st));
-    *codes = p;
-    return RNSM_OK;
-}
-
-// The codes for the prunes: where they are the rows.
-const uint8_t *exact_codes(const Codes &cd) { return cd.mode == kCodeExact ? cd.rows : nullptr; }
 
 // A beam search evaluates some 16 vertices per entry of its beam.
 int64_t search_evals(int64_t queries, int32_t ef) { return 16 * queries * ef; }
@@ -462,7 +444,7 @@ rnsm_status reverse_into(const SegTable &tab, int32_t dim, const rnsm_params &p,
                          const int32_t *eu, const int32_t *ev, int64_t cap,
                          const unsigned long long *count, int32_t key_lo, int64_t nkeys,
                          int32_t csr_max_bound, const RevBufs &r, const Ctl &c, cudaStream_t st,
-                         const QuantBufs *qb = nullptr, const uint8_t *codes = nullptr) {
+                         const QuantBufs *qb = nullptr, const Codes *codes = nullptr) {
     CK(launch_bucket(eu, ev, cap, count, nkeys, key_lo, r.offs, r.cursor, r.ids, r.scan_tmp,
                      r.scan_bytes, st));
     int32_t csr_max = csr_max_bound;
@@ -487,7 +469,7 @@ rnsm_status reverse_into(const SegTable &tab, int32_t dim, const rnsm_params &p,
     a.csr_ids = r.ids;
     a.csr_max = csr_max;
     a.out = lists;
-    a.codes = codes;
+    if (codes) prune_codes(a, *codes, c);
     a.err = c.err;
     apply_quant(a, qb, c.rechecks, c.tile_err, c.tile_tests);
     return run_prune(a, c.work + 6, c, st, 1);
@@ -763,13 +745,16 @@ rnsm_status rnsm_prune(const float *vecs, int64_t n, int32_t dim, const int32_t 
     take_ctl(b, c, nv);
     take_quant(b, n, dim, qprec, metric, qb);
     TRY(ctl_reset(c, st));
-    bool scanned = false;
-    TRY(scan_table(one_table(vecs, n), dim, metric,
-                   prec == RNSM_PREC_FP32 && w_len <= kPruneSmallMax ? nv * w_len : 0, c, st, scanned));
-    CK(launch_validate(scanned ? nullptr : vecs, n * dim, {owners, nv, n, 0}, {pool, nv * w_len, n, -1}, {}, c.err, st));
-    CodeStats rows;
-    const bool gated = qprec == 0 && !scanned && nv <= kGateOwners;   // FP32 kernels: one wait, at the end
-    if (!gated) TRY(check_err_word(c, st, &rows));
+    // coded rows where the call's pools take them and it is large enough to pay
+    Codes codes;
+    CodeParams code_params;
+    const int64_t evals = prec == RNSM_PREC_FP32 && prune_code_ok(dim, metric) && w_len <= kPruneSmallMax ? nv * w_len : 0;
+    const bool coding = evals >= 8 * n;
+    if (coding) TRY(code_table(one_table(vecs, n), dim, metric, 1, evals, c, st, codes, &code_params));
+    CK(launch_validate(coding ? nullptr : vecs, n * dim, {owners, nv, n, 0}, {pool, nv * w_len, n, -1}, {}, c.err, st));
+    const bool gated = qprec == 0 && !coding && nv <= kGateOwners;   // FP32 kernels: one wait, at the end
+    if (!gated) TRY(check_err_word(c, st));
+    if (coding) code_mode(codes, code_params, dim, metric);
     SegTable tab;
     std::memset(&tab, 0, sizeof(tab));
     tab.base[0] = vecs;
@@ -791,7 +776,7 @@ rnsm_status rnsm_prune(const float *vecs, int64_t n, int32_t dim, const int32_t 
     a.out = out;
     a.out_by_index = 1;
     a.err = c.err;
-    TRY(code_scanned(tab, dim, metric, scanned, rows, c, st, &a.codes));
+    prune_codes(a, codes, c);
     if (qb.q) CK(launch_quantize(tab, n, dim, qprec, qb.q, qb.qlo, qb.scale, qb.err, qb.norm, st));
     TRY(pair_exactness(tab, dim, qprec, metric, c, st, qb));
     apply_quant(a, &qb, c.rechecks, nullptr, c.tile_tests);
@@ -821,12 +806,14 @@ rnsm_status rnsm_reverse_edges(const float *vecs, int64_t n, int32_t dim, int32_
     take_ctl(b, c, n);
     take_rev(b, n, ne, r);
     TRY(ctl_reset(c, st));
-    bool scanned = false;
-    TRY(scan_table(one_table(vecs, n), dim, metric, 16 * ne, c, st, scanned));
-    CK(launch_validate(scanned ? nullptr : vecs, n * dim, {lists, n * R, n, -1}, {eu, ne, n, 0}, {ev, ne, n, 0}, c.err,
+    Codes codes;
+    CodeParams code_params;
+    const bool coding = prune_code_ok(dim, metric) && 16 * ne >= 8 * n;
+    if (coding) TRY(code_table(one_table(vecs, n), dim, metric, 1, 16 * ne, c, st, codes, &code_params));
+    CK(launch_validate(coding ? nullptr : vecs, n * dim, {lists, n * R, n, -1}, {eu, ne, n, 0}, {ev, ne, n, 0}, c.err,
                        st));
-    CodeStats rows;
-    TRY(check_err_word(c, st, &rows));
+    TRY(check_err_word(c, st));
+    if (coding) code_mode(codes, code_params, dim, metric);
     SegTable tab;
     std::memset(&tab, 0, sizeof(tab));
     tab.base[0] = vecs;
@@ -837,9 +824,7 @@ rnsm_status rnsm_reverse_edges(const float *vecs, int64_t n, int32_t dim, int32_
     p.R = R;
     p.alpha = alpha;
     p.metric = metric;
-    const uint8_t *codes = nullptr;
-    TRY(code_scanned(tab, dim, metric, scanned, rows, c, st, &codes));
-    TRY(reverse_into(tab, dim, p, lists, eu, ev, ne, nullptr, 0, n, -1, r, c, st, nullptr, codes));
+    TRY(reverse_into(tab, dim, p, lists, eu, ev, ne, nullptr, 0, n, -1, r, c, st, nullptr, &codes));
     TRY(check_err_word(c, st));
     return RNSM_OK;
 }
@@ -957,10 +942,10 @@ rnsm_status rnsm_build_segment(const float *vecs, int64_t n, int32_t dim, const 
         q.ev = ev;
         q.ecount = c.ecount;
         q.err = c.err;
-        q.codes = exact_codes(codes);
+        prune_codes(q, codes, c);
         TRY(run_prune(q, c.work + 8, c, st));
         TRY(reverse_into(tab, dim, p, out_adj, eu, ev, bsz * p.R, c.ecount, 0, n, (int32_t)bsz, r,
-                         c, st, nullptr, exact_codes(codes)));
+                         c, st, nullptr, &codes));
         inserted += bsz;
     }
     TRY(check_err_word(c, st));
@@ -1519,7 +1504,7 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
                 q.out = out_adj;
                 q.err = c.err;
                 apply_quant(q, &mb.qb, c.rechecks, c.tile_err, c.tile_tests);
-                q.codes = exact_codes(codes);
+                prune_codes(q, codes, c);
                 TRY(run_prune(q, c.work + 8, c, es, 0));
             }
             tm.end(span);
@@ -1527,7 +1512,7 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
             CK(cudaMemsetAsync(c.ecount, 0, sizeof(unsigned long long), es));
             CK(launch_emit_cross(out_adj, p.R, tab, mk, mb.eu, mb.ev, c.ecount, es));
             TRY(reverse_into(tab, dim, p, out_adj, mb.eu, mb.ev, tab.off[m] * p.R, c.ecount, 0,
-                             tab.off[m], -1, mb.rev, c, es, &mb.qb, exact_codes(codes)));
+                             tab.off[m], -1, mb.rev, c, es, &mb.qb, &codes));
             CK(cudaMemsetAsync(mb.rev_counts + g0, 0, sizeof(unsigned long long) * (g1 - g0), es));
             CK(cudaMemcpyAsync(mb.rev_counts + g0, c.ecount, sizeof(unsigned long long),
                                cudaMemcpyDeviceToDevice, es));
@@ -1562,13 +1547,13 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
             q.ecount = c.ecount;
             q.err = c.err;
             apply_quant(q, &mb.qb, c.rechecks, c.tile_err, c.tile_tests);
-            q.codes = exact_codes(codes);
+            prune_codes(q, codes, c);
             TRY(run_prune(q, c.work + 8, c, es, 0));
             tm.end(span);
             span = graph ? -1 : tm.begin(7);
             TRY(reverse_into(tab, dim, p, out_adj, mb.eu, mb.ev, ns * p.R, c.ecount, t0, nt,
                              graph ? kReversePoolBound - p.R : -1, mb.rev, c, es, &mb.qb,
-                             exact_codes(codes)));
+                             &codes));
             CK(cudaMemcpyAsync(mb.rev_counts + e, c.ecount, sizeof(unsigned long long),
                                cudaMemcpyDeviceToDevice, es));
             tm.end(span);

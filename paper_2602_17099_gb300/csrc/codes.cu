@@ -12,8 +12,6 @@
 // Rows of integers that span at most 255 (SIFT) have s = 1 and e = 0: S is the
 // squared distance itself, and no FP32 row is needed (kCodeExact).
 #include <float.h>
-#include <math.h>
-#include <string.h>
 
 #include "internal.h"
 
@@ -192,18 +190,6 @@ __global__ void __launch_bounds__(1024) code_final_kernel(const SegTable t, int 
 
 }  // namespace
 
-// Whether the scanned rows are their codes (code_grid's s = 1).
-bool codes_exact(const CodeStats &s) {
-    auto value = [](uint32_t u) {
-        const uint32_t b = (u & 0x80000000u) ? u ^ 0x80000000u : ~u;
-        float f;
-        memcpy(&f, &b, sizeof(f));
-        return f;
-    };
-    const float a = value(~s.omin_inv), b = value(s.omax);
-    return !s.fraction && b - a <= 255.f && fabsf(a) <= 65536.f;
-}
-
 bool codes_dim_ok(int dim) { return dim == 64 || dim == 96 || dim == 128 || dim == 256 || dim == 768; }
 
 cudaError_t launch_code_scan(const SegTable &t, int32_t dim, int32_t checked, CodeStats *s, int32_t *err,
@@ -220,10 +206,8 @@ cudaError_t launch_code_rows(const SegTable &t, int32_t dim, int32_t metric, uin
     int64_t g = (t.off[t.m] + 7) / 8;
     if (g > 152 * 8) g = 152 * 8;
     code_rows_kernel<<<(unsigned)(g < 1 ? 1 : g), 256, 0, st>>>(t, dim, codes, s);
-    note_launches(1);
-    if (!p) return cudaGetLastError();
     code_final_kernel<<<1, 1024, 0, st>>>(t, dim, metric, s, p);
-    note_launches(1);
+    note_launches(2);
     return cudaGetLastError();
 }
 

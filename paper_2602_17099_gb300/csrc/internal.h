@@ -59,10 +59,8 @@ bool codes_dim_ok(int dim);
 // the statistics, in one pass over the table's rows; then the codes (rows by global id) and the constants.
 cudaError_t launch_code_scan(const SegTable &t, int32_t dim, int32_t checked, CodeStats *s, int32_t *err,
                              cudaStream_t st);
-// (p null: no constants.)
 cudaError_t launch_code_rows(const SegTable &t, int32_t dim, int32_t metric, uint8_t *codes, CodeStats *s,
                              CodeParams *p, cudaStream_t st);
-bool codes_exact(const CodeStats &s);
 // Launches of up to this many queries take the search's latency shape, which
 // does not filter by codes.
 constexpr int64_t kLatencyQueries = 1216;
@@ -191,7 +189,8 @@ struct PruneArgs {
     unsigned long long *ovf_count;
     int32_t *err;             // bit 4: pool larger than the capacity; bit 6: tile wait ran out
     int32_t test_withhold_commit;  // test-only (tensor-core prune): never signal MMA completion
-    const uint8_t *codes;     // nullable: exact coded rows by global id (codes.cu)
+    const uint8_t *codes;     // nullable: coded rows by global id (codes.cu)
+    const CodeParams *code_params;   // their constants; null: the codes are the rows
     int32_t pair_hi_only;     // pair tile: integer rows spanning <= 256, hi terms only
 };
 
@@ -207,7 +206,7 @@ cudaError_t launch_small(const PruneArgs &a, cudaStream_t st);
 // The same pools (d <= kPruneWalkMaxDim) by the walk over kept rows only.
 constexpr int kPruneWalkMaxDim = 128;
 cudaError_t launch_walk(const PruneArgs &a, cudaStream_t st);
-// The same pools where the rows are exact codes (a.codes; L2, d = 64, 96, 128).
+// The same pools over coded rows (a.codes; L2, d = 64, 96, 128).
 bool prune_code_ok(int dim, int metric);
 cudaError_t launch_prune_code(const PruneArgs &a, cudaStream_t st);
 cudaError_t launch_prune_general(const PruneArgs &a, const int32_t *idx_list,

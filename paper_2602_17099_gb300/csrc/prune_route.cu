@@ -21,8 +21,8 @@ namespace {
 //             stored BF16 / E4M3 terms);
 //   kVarFp32: the FP32 kernels (register-blocked triangle for pools <= 64);
 //   kVarWalk: the FP32 walk over kept rows (pools <= 64, d <= 128);
-//   kVarCode: the walk over exact coded rows (pools <= 64; where the call has them:
-//             integer rows, L2, d = 64, 96, 128).
+//   kVarCode: the walk over coded rows (pools <= 64, L2, d = 64, 96, 128, where the
+//             call has them; tests that they leave open are decided in FP32).
 enum { kVarFp32 = 0, kVarPair = 1, kVarTile = 2, kVarWalk = 3, kVarCode = 4, kVarCount = 5 };
 
 int forced_prune_variant() {
@@ -64,7 +64,7 @@ cudaError_t run_variant(const PruneArgs &a, int var, cudaStream_t st) {
 // The variants that apply to a call, the default (the first) included.
 int variants_of(const PruneArgs &a, int *out) {
     int n = 0;
-    // exact coded rows: a quarter of the bytes and an eighth of the instructions of
+    // coded rows: a quarter of the bytes and an eighth of the instructions of
     // FP32 rows (2 x 500k SIFT-like rows, S6 + S7: 4.8 ms; the FP32 walk 23.0, the
     // BF16 pair tile 12.5, the FP8 one 14.7), so in FP32 mode nothing else is tried.
     // With tiles asked for they are one of the tuner's choices, not the default.
