@@ -645,6 +645,8 @@ def run_ours(args, ws, rank, local):
                   "flop_per_owner_at_most": W.R * pool * W.dim * 2,
                   # measured: the FMA pipe's activity in the committed ncu capture
                   "fma_pipe_active_pct_ncu": prune_profile_fma(s6_var) if W.name == "sift2x500k" else None}
+    if s6_var == 4:   # integer dot products of coded rows: no FP32 arithmetic to rate
+        prune_flop = None
     # the dominant kernel family of the FP32 step by live time goes first
     s7_ms = sum(st["phase_ms"][7] for st in stats)
     if p_ms + s7_ms >= s_ms:

@@ -16,9 +16,9 @@
 //
 // 2 x 500k SIFT-like rows (exact, d = 128): S6 13.3 -> 2.40 ms, S7 9.7 -> 2.43 ms
 // (twenty warps per SM; 16 with registers to spare: 2.47 ms).  DEEP-like rows
-// (filter, d = 96): 100k owners, pools of 64, 2.82 -> 1.42 ms (16 warps per SM; 20 with
-// spills: 1.74), 1.6 M reverse edges into 150k lists 2.70 -> 2.35 ms.  There the FP32 rows
-// of the owner distances, a row a lane, fill two thirds of the L1 pipe.
+// (filter, d = 96): 100k owners, pools of 64, 2.82 -> 1.16 ms (16 warps per SM; 20 with
+// spills: 1.15, and a graph build 8 % slower), 1.6 M reverse edges into 150k lists
+// 2.70 -> 1.98 ms.
 //
 // Per owner (one warp): the rows by cp.async into shared memory; every lane its
 // two candidates' distances to the owner; positions by counting (64-bit keys of
@@ -45,35 +45,11 @@ struct CodePool {
     int32_t id[kPool];
     int32_t slot[kPool];               // filter: raw slot of each position
     float4 vrow[kExact ? 1 : W];       // filter: the owner's FP32 row
+    const float *rptr[kExact ? 1 : kPool];   // filter: FP32 row of each slot, null: none
 };
 
 template <int W, bool kExact>
 constexpr int code_blocks() { return (W == 32 ? 5 : W == 24 ? 6 : 8) - (kExact ? 0 : 2); }
-
-// The FP32 prune distances of the owner to rows x0 and x1 (x1 null: none), the
-// chain of prune_dist; both rows' loads kAhead float4 ahead.
-template <int W>
-__device__ __forceinline__ void owner_dists(const float4 *v, const float *x0, const float *x1, float &d0, float &d1) {
-    constexpr int kAhead = W == 24 ? 6 : 4;
-    f2_t a0 = 0ull, a1 = 0ull;
-#pragma unroll 1
-    for (int f = 0; f < W; f += kAhead) {
-        ulonglong2 p[kAhead], q[kAhead];
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u) {
-            p[u] = ldg_u2(x0 + 4 * (f + u));
-            if (x1) q[u] = ldg_u2(x1 + 4 * (f + u));
-        }
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u) {
-            const ulonglong2 o = *reinterpret_cast<const ulonglong2 *>(v + f + u);
-            a0 = chain2(a0, o, p[u], 0);
-            if (x1) a1 = chain2(a1, o, q[u], 0);
-        }
-    }
-    d0 = chain2_final(a0, 0);
-    if (x1) d1 = chain2_final(a1, 0);
-}
 
 // The FP32 distance of two rows by id: the few tests that the codes leave open.  Not
 // inlined: its loads would cost the walk registers, and with them warps.
@@ -107,6 +83,40 @@ __device__ __forceinline__ void cp_async16(uint32_t *dst, const uint8_t *src) {
                      static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
                  "l"(src)
                  : "memory");
+}
+
+// The FP32 prune distances of the owner to this lane's two rows, the chain of
+// prune_dist.  The rows pass through s.rows a quarter at a time (a quarter is as long as
+// a code row): copied by consecutive lanes, read back a row a lane.  Loaded a row a
+// lane straight from global memory, each 16-byte load of a warp touched 32 lines, and
+// the L1 pipe was the kernel's limit (100k DEEP-like owners 1.41 ms, now 1.16).
+template <int W, class Pool>
+__device__ __forceinline__ void owner_dists(Pool &s, int nr, bool two, float &d0, float &d1) {
+    constexpr int kStride = Pool::kStride, kVec = W / 4;
+    const int lane = threadIdx.x & 31;
+    f2_t a0 = 0ull, a1 = 0ull;
+#pragma unroll 1
+    for (int c = 0; c < 4; ++c) {
+        for (int u = lane; u < nr * kVec; u += 32) {
+            const int r = u / kVec, f = u - r * kVec;
+            const float *x = s.rptr[r];
+            if (x) cp_async16(s.rows + r * kStride + 4 * f, reinterpret_cast<const uint8_t *>(x + c * W + 4 * f));
+        }
+        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+        __syncwarp();
+        const ulonglong2 *v = reinterpret_cast<const ulonglong2 *>(s.vrow + c * kVec);
+        const ulonglong2 *x0 = reinterpret_cast<const ulonglong2 *>(s.rows + lane * kStride);
+        const ulonglong2 *x1 = reinterpret_cast<const ulonglong2 *>(s.rows + (lane + 32) * kStride);
+#pragma unroll
+        for (int f = 0; f < kVec; ++f) {
+            const ulonglong2 o = v[f];
+            a0 = chain2(a0, o, x0[f], 0);
+            if (two) a1 = chain2(a1, o, x1[f], 0);
+        }
+        __syncwarp();
+    }
+    d0 = chain2_final(a0, 0);
+    if (two) d1 = chain2_final(a1, 0);
 }
 
 template <int W, bool kExact>
@@ -162,28 +172,24 @@ __global__ void __launch_bounds__(kCodeWarps * 32, code_blocks<W, kExact>())
                 }
                 id[h] = c;
                 s.id[j] = c;
+                if (!kExact) s.rptr[j] = c >= 0 ? seg_row(a.segs, c, 4 * W) : nullptr;
+            }
+            const bool two = nr > 32;
+            float e0 = INFINITY, e1 = INFINITY;   // filter: FP32 distances to the owner
+            if (!kExact) {   // the order is that of the FP32 chain
+                const float *orow = seg_row(a.segs, owner, 4 * W);
+                if (lane < W) s.vrow[lane] = ldg4(orow + 4 * lane);
+                __syncwarp();
+                owner_dists<W>(s, nr, two, e0, e1);
             }
             __syncwarp();
-            const float *orow = nullptr;
-            if (!kExact) {
-                orow = seg_row(a.segs, owner, 4 * W);
-                if (lane < W) s.vrow[lane] = ldg4(orow + 4 * lane);
-            } else if (lane < kVec) cp_async16(s.owner + 4 * lane, a.codes + (int64_t)owner * (4 * W) + 16 * lane);
+            if (kExact && lane < kVec) cp_async16(s.owner + 4 * lane, a.codes + (int64_t)owner * (4 * W) + 16 * lane);
             for (int c = lane; c < nr * kVec; c += 32) {
                 const int r = c / kVec, f = c - r * kVec;
                 const int32_t g = s.id[r];
                 if (g >= 0) cp_async16(s.rows + r * kStride + 4 * f, a.codes + (int64_t)g * (4 * W) + 16 * f);
             }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            const bool two = nr > 32;
-            float e0 = INFINITY, e1 = INFINITY;   // filter: FP32 distances to the owner
-            if (!kExact) {
-                // while the codes are on their way: the order is that of the FP32 chain
-                __syncwarp();
-                owner_dists<W>(s.vrow, seg_row(a.segs, id[0] >= 0 ? id[0] : owner, 4 * W),
-                               two ? seg_row(a.segs, id[1] >= 0 ? id[1] : owner, 4 * W) : nullptr, e0, e1);
-            }
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
             __syncwarp();
             // 2. keys: distance to the owner, id, slot (none repeats)
             uint32_t nv = 0u, n0 = 0u, n1 = 0u, v0 = 0u, v1 = 0u;
