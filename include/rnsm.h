@@ -172,7 +172,8 @@ typedef struct {
      * on the owner distances of every 64th owner: [0] max |d~ - d64| / d64
      * (tile vs FP64), [1] max |d32 - d64| / d64 (the FP32 distance vs FP64),
      * [2] max |d~ - d32| / B (the share of its error bound B the tile used),
-     * [3] number of distances sampled.  Zero in FP32 mode. */
+     * [3] number of distances sampled.  Zero in FP32 mode and where no tile ran
+     * (prune_kernel: larger calls may take another variant). */
     double tile_error[4];
     /* BF16 / FP8 modes: occlusion tests the tensor-core tiles evaluated (the
      * share that was re-decided is rechecks / tile_tests, owner-distance

@@ -61,18 +61,21 @@ cudaError_t run_variant(const PruneArgs &a, int var, cudaStream_t st) {
     return launch_prune_general(b, a.ovf_list, a.ovf_count, st);
 }
 
+constexpr int64_t kCodeFirst = 16384;
+
 // The variants that apply to a call, the default (the first) included.
 int variants_of(const PruneArgs &a, int *out) {
     int n = 0;
-    // coded rows: a quarter of the bytes and an eighth of the instructions of
-    // FP32 rows (2 x 500k SIFT-like rows, S6 + S7: 4.8 ms; the FP32 walk 23.0, the
-    // BF16 pair tile 12.5, the FP8 one 14.7), so in FP32 mode nothing else is tried.
-    // With tiles asked for they are one of the tuner's choices, not the default.
+    // coded rows: a quarter of the bytes and an eighth of the instructions of FP32 rows,
+    // so in FP32 mode nothing else is tried (2 x 500k SIFT-like rows, S6 + S7: 4.8 ms; the
+    // FP32 walk 23.0, the BF16 pair tile 12.5, the FP8 one 14.7.  100k DEEP-like owners: 1.16
+    // ms; the FP32 walk 2.82).  With tiles asked for they come first from kCodeFirst owners
+    // on (300k DEEP-like rows in 6 plan edges, S6 + S7: 8.0 ms, the BF16 pair tile 11.8);
+    // below that the launch is short either way and the tiles stay the default.
     const bool code_ok = a.codes && prune_code_ok(a.dim, a.metric) && a.lenA + a.lenB <= kPruneSmallMax;
-    if (code_ok && a.prec == 0) {
-        out[n++] = kVarCode;
-        if (forced_prune_variant() < 0) return n;
-    }
+    const bool code_first = code_ok && (a.prec == 0 || a.n_owners >= kCodeFirst);
+    if (code_first) out[n++] = kVarCode;
+    if (code_first && a.prec == 0 && forced_prune_variant() < 0) return n;
     if (a.prec != 0) {
         const bool pair_ok = prune_pair_ok(a.dim, a.prec, a.metric);
         if (pair_ok && a.lenA + a.lenB <= prune_pair_max_pool()) out[n++] = kVarPair;
@@ -82,7 +85,7 @@ int variants_of(const PruneArgs &a, int *out) {
             a.lenA + a.lenB <= prune_tc_max_pool())
             out[n++] = kVarTile;
     }
-    if (code_ok && a.prec != 0) out[n++] = kVarCode;
+    if (code_ok && !code_first) out[n++] = kVarCode;
     // FP32 defaults (calls too small to tune): the walk for the source pools, the
     // triangle for reverse-edge pools (on deep-like rows the walk lost there by 40 %)
     const bool walk_ok = a.dim <= kPruneWalkMaxDim && a.lenA + a.lenB <= kPruneSmallMax;
