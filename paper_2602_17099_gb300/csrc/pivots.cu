@@ -27,10 +27,10 @@
 //
 // The uncovered vertices are listed anew every round, and the last rounds, few
 // vertices each, run in one launch of one thread-block cluster, which needs no host
-// between rounds (all rounds of up to kTailMax vertices run there; with 6 rounds over
-// the whole grid before it instead of 16, 500k rows left it 1.5 ms of work).  What is
-// left is the chain of dependent loads of each round, some 14 us.  S3 of 5,000
-// Gaussian rows 2.14 -> 0.55 ms, 2 x 500k SIFT-like rows 1.55 -> 0.81 ms, 300k
+// between rounds (all rounds of up to kTailMax vertices run there, of up to kSmallMax in
+// one block; with 6 rounds over the whole grid before it instead of 16, 500k rows left
+// it 1.5 ms of work).  What is left is the chain of dependent loads of each round, some
+// 11 us.  S3 of 5,000 Gaussian rows 2.14 -> 0.41 ms, 2 x 500k SIFT-like rows 1.55 -> 0.81 ms, 300k
 // DEEP-like rows in 5 segments 3.25 -> 1.90 ms.
 
 #include <cooperative_groups.h>
@@ -45,6 +45,7 @@ constexpr int32_t kCovered = -(1 << 30);   // gain of a covered vertex (and belo
 constexpr int64_t kTailMax = 32768;
 constexpr int kWide = 24;                  // reverse lists from here on take a warp
 constexpr int kFullRounds = 16;            // rounds over the whole grid before the cluster's
+constexpr int64_t kSmallMax = 6144;        // 16 bytes of state each in one block's shared memory
 constexpr int kTailBlocks = 8, kTailThreads = 1024;
 
 struct PivotState {
@@ -72,23 +73,37 @@ __global__ void piv_init_kernel(PivotState s, int64_t n, int32_t *list, PivotCtl
     }
 }
 
+// The state lies in global memory (read past L1: other blocks write it) or, for the
+// one-block kernel, in shared memory with 16-bit lists.
+template <bool kShared, class T>
+__device__ __forceinline__ int32_t get(const T *p) {
+    if constexpr (kShared) return (int32_t)*const_cast<const volatile T *>(p);
+    else return __ldcg(p);
+}
+template <bool kShared, class T>
+__device__ __forceinline__ void put(T *p, int32_t v) {
+    if constexpr (kShared) *const_cast<volatile T *>(p) = (T)v;
+    else __stcg(p, v);
+}
+
 // Lists the uncovered vertices of cur[0..nc) in next and takes their votes;
 // thread t of `threads` (whole warps).
-__device__ __forceinline__ void vote_phase(const PivotState &s, const int32_t *cur, int32_t nc, int32_t *next,
-                                           int32_t *n_next, int64_t t, int64_t threads) {
+template <bool kShared, class T>
+__device__ __forceinline__ void vote_phase(const PivotState &s, const T *cur, int32_t nc, T *next, int32_t *n_next,
+                                           int64_t t, int64_t threads) {
     const int lane = threadIdx.x & 31;
     for (int64_t i0 = t - lane; i0 < nc; i0 += threads) {
         const int64_t i = i0 + lane;
-        const int32_t z = i < nc ? __ldcg(cur + i) : -1;
-        const int32_t gz = z >= 0 ? __ldcg(s.gain + z) : kCovered;
+        const int32_t z = i < nc ? get<kShared>(cur + i) : -1;
+        const int32_t gz = z >= 0 ? get<kShared>(s.gain + z) : kCovered;
         const bool open = gz >= 0;
         const unsigned m = __ballot_sync(0xffffffffu, open);
         int base = 0;
         if (lane == 0 && m) base = atomicAdd(n_next, __popc(m));
         base = __shfl_sync(0xffffffffu, base, 0);
         if (!open) continue;
-        __stcg(next + base + __popc(m & lanemask_lt()), z);
-        __stcg(s.snap + z, gz);
+        put<kShared>(next + base + __popc(m & lanemask_lt()), z);
+        put<kShared>(s.snap + z, gz);
         int32_t best = z, gb = gz;
         int weight = 1;   // z's own
         const int32_t *nz = s.nplus + (int64_t)z * s.k_plus;
@@ -96,7 +111,7 @@ __device__ __forceinline__ void vote_phase(const PivotState &s, const int32_t *c
         for (int j = 0; j < s.k; ++j) {
             const int32_t y = __ldg(nz + j);
             if (y < 0) continue;
-            const int32_t gy = __ldcg(s.gain + y);
+            const int32_t gy = get<kShared>(s.gain + y);
             if (y == best) ++weight;
             else if (gy > gb || (gy == gb && gy >= 0 && y < best)) {
                 best = y;
@@ -108,16 +123,38 @@ __device__ __forceinline__ void vote_phase(const PivotState &s, const int32_t *c
     }
 }
 
-// Covers entry e of the selected x's reverse list (e = lo - 1: x itself).
-__device__ __forceinline__ void cover(const PivotState &s, int32_t x, int64_t e, int64_t lo) {
-    const int32_t y = e < lo ? x : s.ids[e];
-    if (e >= lo && (y == x || __ldcg(s.gain + y) < 0)) return;
-    if (atomicExch(s.gain + y, kCovered) < 0) return;   // listed twice: once
-    __stcg(s.pivot_of + y, e < lo ? -1 : x);
-    const int32_t *ny = s.nplus + (int64_t)y * s.k_plus;
-    for (int c = 0; c < s.k; ++c) {
-        const int32_t w = __ldg(ny + c);
-        if (w >= 0) atomicSub(s.gain + w, 1);
+// Covers the selected x and its uncovered reverse neighbours, by G lanes; four entries
+// a lane at a time, so that a long list is not a chain of one entry's loads after
+// another's (entry lo - 1: x itself).
+template <bool kShared, int G>
+__device__ __forceinline__ void cover_list(const PivotState &s, int32_t x, int64_t lo, int64_t hi, int sub) {
+    for (int64_t e0 = lo + sub - 1; e0 < hi; e0 += 4 * G) {
+        int32_t y[4];
+        bool todo[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t e = e0 + q * G;
+            y[q] = e >= hi ? -1 : e < lo ? x : __ldg(s.ids + e);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const bool self = q == 0 && e0 < lo;
+            todo[q] = self || (y[q] >= 0 && y[q] != x && get<kShared>(s.gain + y[q]) >= 0);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)   // (a vertex listed twice: once)
+            if (todo[q]) todo[q] = atomicExch(s.gain + y[q], kCovered) >= 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (todo[q]) __stcg(s.pivot_of + y[q], q == 0 && e0 < lo ? -1 : x);
+        for (int c = 0; c < s.k; ++c) {
+            int32_t w[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) w[q] = todo[q] ? __ldg(s.nplus + (int64_t)y[q] * s.k_plus + c) : -1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (w[q] >= 0) atomicSub(s.gain + w[q], 1);
+        }
     }
 }
 
@@ -130,16 +167,16 @@ __device__ __forceinline__ unsigned drop_lowest(unsigned m, int n) {
 // pivots, their uncovered reverse neighbours followers.  Eight lanes per
 // selected vertex, a warp where the reverse list is long (a hub's list by eight
 // lanes is a chain of |R_k| / 8 rounds of four dependent loads).
-__device__ __forceinline__ void select_phase(const PivotState &s, const int32_t *next, int32_t n, int64_t t,
-                                             int64_t threads) {
+template <bool kShared, class T>
+__device__ __forceinline__ void select_phase(const PivotState &s, const T *next, int32_t n, int64_t t, int64_t threads) {
     const int lane = threadIdx.x & 31, sub = lane & 7, grp = lane >> 3;
     for (int64_t i0 = t - lane; i0 < n; i0 += threads) {
         const int64_t i = i0 + lane;
-        const int32_t x = i < n ? __ldcg(next + i) : -1;
+        const int32_t x = i < n ? get<kShared>(next + i) : -1;
         bool sel = false;
         if (x >= 0) {
-            sel = __ldcg(s.votes + x) == __ldcg(s.snap + x) + 1;
-            __stcg(s.votes + x, 0);
+            sel = get<kShared>(s.votes + x) == get<kShared>(s.snap + x) + 1;
+            put<kShared>(s.votes + x, 0);
         }
         int64_t lo = 0, hi = 0;
         if (sel) {
@@ -153,15 +190,14 @@ __device__ __forceinline__ void select_phase(const PivotState &s, const int32_t 
             const int src = r ? __ffs(r) - 1 : lane;
             const int32_t xs = __shfl_sync(0xffffffffu, x, src);
             const int64_t l = __shfl_sync(0xffffffffu, lo, src), h = __shfl_sync(0xffffffffu, hi, src);
-            if (r)
-                for (int64_t e = l + sub - 1; e < h; e += 8) cover(s, xs, e, l);
+            if (r) cover_list<kShared, 8>(s, xs, l, h, sub);
             __syncwarp();
         }
         for (m = __ballot_sync(0xffffffffu, wide); m; m &= m - 1u) {
             const int src = __ffs(m) - 1;
             const int32_t xs = __shfl_sync(0xffffffffu, x, src);
             const int64_t l = __shfl_sync(0xffffffffu, lo, src), h = __shfl_sync(0xffffffffu, hi, src);
-            for (int64_t e = l + lane - 1; e < h; e += 32) cover(s, xs, e, l);
+            cover_list<kShared, 32>(s, xs, l, h, lane);
             __syncwarp();
         }
     }
@@ -169,14 +205,14 @@ __device__ __forceinline__ void select_phase(const PivotState &s, const int32_t 
 
 __global__ void __launch_bounds__(256) piv_vote_kernel(PivotState s, const int32_t *cur, int32_t *next, PivotCtl *ctl,
                                                        int round) {
-    vote_phase(s, cur, ctl->count[round], next, &ctl->count[round + 1], blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
+    vote_phase<false>(s, cur, ctl->count[round], next, &ctl->count[round + 1], blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
                (int64_t)gridDim.x * blockDim.x);
 }
 
 __global__ void __launch_bounds__(256) piv_select_kernel(PivotState s, const int32_t *next, PivotCtl *ctl, int round) {
     const int32_t n = ctl->count[round + 1];
     if (n > 0 && blockIdx.x == 0 && threadIdx.x == 0) ++ctl->rounds;
-    select_phase(s, next, n, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+    select_phase<false>(s, next, n, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
 // The remaining rounds, by one cluster.  Each round has fewer uncovered vertices
@@ -189,7 +225,7 @@ __global__ void __cluster_dims__(kTailBlocks, 1, 1) __launch_bounds__(kTailThrea
     int32_t *slot = &ctl->count[round];   // slot[1], slot[2], slot[3] take turns
     for (int r = 0;; ++r) {
         int32_t *n_next = slot + 1 + r % 3;
-        vote_phase(s, cur, nc, next, n_next, t, threads);
+        vote_phase<false>(s, cur, nc, next, n_next, t, threads);
         cluster.sync();
         nc = __ldcg(n_next);
         if (nc == 0) break;
@@ -200,13 +236,78 @@ __global__ void __cluster_dims__(kTailBlocks, 1, 1) __launch_bounds__(kTailThrea
         before = nc;
         ++rounds;
         if (t == 0) __stcg(slot + 1 + (r + 2) % 3, 0);   // next but one: read by all a round ago
-        select_phase(s, next, nc, t, threads);
+        select_phase<false>(s, next, nc, t, threads);
         cluster.sync();
         int32_t *sw = cur;
         cur = next;
         next = sw;
     }
     if (t == 0) ctl->rounds += rounds;
+}
+
+// All of it for up to kSmallMax vertices, by one block with the state in shared memory:
+// a round's chain of dependent accesses then mostly costs tens of cycles instead of
+// hundreds each (5,000 Gaussian rows, 32 rounds: 464 us by the cluster, now 340; 8,001
+// DEEP-like rows: the cluster is faster by 30 us).
+__global__ void __launch_bounds__(kTailThreads) piv_small_kernel(PivotState s, int32_t n, int32_t *pivots,
+                                                                 int32_t *followers, PivotCtl *ctl) {
+    extern __shared__ int32_t state[];
+    __shared__ int32_t cnt[3], n_piv, n_fol;
+    s.gain = state;
+    s.votes = state + n;
+    s.snap = state + 2 * n;
+    uint16_t *cur = reinterpret_cast<uint16_t *>(state + 3 * n), *next = cur + n;
+    const int t = threadIdx.x, lane = t & 31;
+    for (int x = t; x < n; x += kTailThreads) {
+        s.gain[x] = (int32_t)(s.offs[x + 1] - s.offs[x]);
+        s.votes[x] = 0;
+        cur[x] = (uint16_t)x;
+    }
+    if (t < 3) cnt[t] = 0;
+    if (t == 0) n_piv = n_fol = 0;
+    __syncthreads();
+    int32_t nc = n, before = INT32_MAX, rounds = 0, stuck = 0;
+    for (int r = 0;; ++r) {
+        vote_phase<true>(s, cur, nc, next, &cnt[r % 3], t, kTailThreads);
+        __syncthreads();
+        nc = cnt[r % 3];
+        if (nc == 0) break;
+        if (nc >= before) {
+            stuck = 1;
+            break;
+        }
+        before = nc;
+        ++rounds;
+        if (t == 0) cnt[(r + 2) % 3] = 0;   // read by all a round ago
+        select_phase<true>(s, next, nc, t, kTailThreads);
+        __syncthreads();
+        uint16_t *sw = cur;
+        cur = next;
+        next = sw;
+    }
+    __syncthreads();   // (pivot_of is this block's own writing)
+    for (int x0 = t - lane; x0 < n; x0 += kTailThreads) {
+        const int x = x0 + lane;
+        const bool pv = x < n && s.pivot_of[x] == -1, fl = x < n && !pv;
+        const unsigned mp = __ballot_sync(0xffffffffu, pv), mf = __ballot_sync(0xffffffffu, fl);
+        int bp = 0, bf = 0;
+        if (lane == 0) {
+            bp = atomicAdd(&n_piv, __popc(mp));
+            bf = atomicAdd(&n_fol, __popc(mf));
+        }
+        bp = __shfl_sync(0xffffffffu, bp, 0);
+        bf = __shfl_sync(0xffffffffu, bf, 0);
+        if (pv) pivots[bp + __popc(mp & lanemask_lt())] = x;
+        if (fl) followers[bf + __popc(mf & lanemask_lt())] = x;
+    }
+    __syncthreads();
+    if (t == 0) {
+        *ctl = PivotCtl();
+        ctl->n_pivots = (unsigned long long)n_piv;
+        ctl->n_followers = (unsigned long long)n_fol;
+        ctl->rounds = rounds;
+        ctl->stuck = stuck;
+    }
 }
 
 __global__ void piv_compact_kernel(int64_t n, const int32_t *pivot_of, int32_t *pivots, int32_t *followers,
@@ -252,6 +353,15 @@ cudaError_t launch_select_pivots(const int32_t *nplus, int64_t n, int32_t k_plus
     s.ids = ids;
     s.k_plus = k_plus;
     s.k = k;
+    if (n <= kSmallMax) {
+        const int smem = (int)(n * (3 * sizeof(int32_t) + 2 * sizeof(uint16_t)));
+        const cudaError_t e = cudaFuncSetAttribute(piv_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)(kSmallMax * 16));
+        if (e != cudaSuccess) return e;
+        piv_small_kernel<<<1, kTailThreads, smem, st>>>(s, (int32_t)n, pivots, followers, ctl);
+        note_launches(1);
+        return cudaGetLastError();
+    }
     // the output lists hold the uncovered vertices meanwhile
     int32_t *cur = pivots, *next = followers;
     const int g = grid_n(n);

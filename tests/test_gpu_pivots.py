@@ -1,5 +1,5 @@
 """Pivot selection on the device against the host's lazy greedy, around the
-sizes where its rounds move from one thread-block cluster to the whole grid,
+sizes where its rounds move from one block to a cluster and to the whole grid,
 with short and long reverse lists (a warp each from 24 entries on), holes and
 the smallest k."""
 import numpy as np
@@ -36,7 +36,7 @@ def _nplus(kind, n, kp, rng):
     return nb.astype(np.int32)
 
 
-@pytest.mark.parametrize("n,k,k_plus", [(7, 2, 2), (1000, 3, 5), (32768, 5, 16), (32769, 5, 16),
+@pytest.mark.parametrize("n,k,k_plus", [(7, 2, 2), (1000, 3, 5), (6144, 5, 16), (6145, 4, 8), (32768, 5, 16), (32769, 5, 16),
                                         (150_001, 7, 7), (90_000, 1, 3)])
 @pytest.mark.parametrize("kind", ["random", "near", "hubs"])
 def test_pivots_equal_the_lazy_greedy(rn, kind, n, k, k_plus):
