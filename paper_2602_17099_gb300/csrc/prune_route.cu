@@ -127,7 +127,9 @@ constexpr int64_t kPruneTuneMinChunk = 20000;   // owners per slice: short launc
 constexpr int64_t kPruneTuneMinEntries = 100000;   // reverse-edge pools: incoming entries
 struct PruneKey {
     int prec, dim, metric, len, csr, site;
+    int codes;   // 0 the call has none, 1 exact, 2 a filter: a choice holds for its like only
     bool operator<(const PruneKey &o) const {
+        if (codes != o.codes) return codes < o.codes;
         if (site != o.site) return site < o.site;
         if (prec != o.prec) return prec < o.prec;
         if (dim != o.dim) return dim < o.dim;
@@ -163,7 +165,8 @@ cudaError_t launch_prune(const PruneArgs &a, cudaStream_t st, int *variant) {
         for (int k = 0; k < nv; ++k)
             if (vars[k] == forced) return run(a, forced);
     if (nv == 1) return run(a, vars[0]);
-    const PruneKey key{a.prec, a.dim, a.metric, a.lenA + a.lenB, a.csr_offs != nullptr, a.tune_site};
+    const PruneKey key{a.prec, a.dim, a.metric, a.lenA + a.lenB, a.csr_offs != nullptr, a.tune_site,
+                       !a.codes ? 0 : a.code_params ? 2 : 1};
     {
         std::lock_guard<std::mutex> lk(g_ptune_mu);
         auto it = g_ptuned.find(key);

@@ -95,3 +95,30 @@ def test_coded_prune_call_equals_fp32(rn, monkeypatch, kind, d, w):
     for mode in ("1", "2"):
         for a, b in zip(res["0"], res[mode]):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("prec", [1, 2])
+def test_tile_modes_take_the_coded_walk_on_large_calls(rn, prec):
+    rng = np.random.default_rng(3)
+    X = torch.from_numpy(_real("unit", 33_500, 96, rng)).cuda()
+    segs = [(x, *rn.build_segment(x, 16, 32)) for x in (X[:16_384].clone(), X[16_384:].clone())]
+    want, _ = rn.merge(segs, rn.params(16, 32))
+    got, st = rn.merge(segs, rn.params(16, 32, prec=prec))
+    assert st["prune_kernel"] == [4, 4]
+    assert torch.equal(got, want)
+
+
+def test_a_tuned_choice_of_codes_does_not_outlive_them(rn, monkeypatch):
+    # calls large enough to tune, in BF16 mode: with codes (the tuner may choose them),
+    # then without, the shape the same
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    X = torch.randn(2000, 64, generator=g, device="cuda")
+    X = X[torch.randint(0, 2000, (490_000,), generator=g, device="cuda")]
+    X = X + 0.5 * torch.randn(X.shape, generator=g, device="cuda")
+    segs = [(x.contiguous(), *rn.build_segment(x.contiguous(), 16, 24)) for x in torch.split(X, 245_000)]
+    first, _ = rn.merge(segs, rn.params(16, 24, prec=1))
+    monkeypatch.setenv("RNSM_SEARCH_CODES", "0")
+    second, st = rn.merge(segs, rn.params(16, 24, prec=1))
+    assert 4 not in st["prune_kernel"]
+    assert torch.equal(first, second)
