@@ -8,8 +8,6 @@ namespace rnsm {
 
 constexpr int kWarp = 32;
 constexpr int kMaxSeg = 64;          // segments addressable by one merge
-constexpr int32_t kExpandedBit = int32_t(0x80000000u);
-constexpr int32_t kIdMask = 0x7fffffff;
 
 // Global id -> row pointer over up to kMaxSeg separately allocated segments.
 struct SegTable {
@@ -54,17 +52,6 @@ __device__ __forceinline__ void warp_sort32(float &d, int32_t &id) {
             if (take) { d = od; id = oi; }
         }
     }
-}
-
-// Number of entries of sorted (sd, si)[0..n) that are lex-less than (d, id).
-__device__ __forceinline__ int lower_bound_lex(const float *sd, const int32_t *si, int n,
-                                               float d, int32_t id) {
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (lex_less(sd[mid], si[mid] & kIdMask, d, id)) lo = mid + 1; else hi = mid;
-    }
-    return lo;
 }
 
 __device__ __forceinline__ void prefetch_l2(const void *p) {

@@ -1,13 +1,8 @@
 // Kernel templates and launchers of K1, the batched beam search; included by
-// the two translation units that instantiate them (single-job launches in
-// search.cu, multi-job launches in search_jobs.cu, compiled in parallel).
+// the translation units that instantiate them (with or without a job table, by
+// code mode; compiled in parallel).
 #pragma once
 #include <float.h>
-#include <stdlib.h>
-
-#include <map>
-#include <mutex>
-#include <utility>
 
 #include "internal.h"
 
@@ -19,10 +14,11 @@ constexpr int kSearchWarps = 4;
 constexpr int kBatch = 32;      // candidates evaluated per batch, one per lane
 
 // Launch-shape variants (identical results): 0 = half the rows in flight and
-// registers capped for 8 CTAs per SM; 1 = the full rows in flight, 5 CTAs;
-// 2 = a whole batch of rows in flight (as far as 128 registers hold it), 2
-// CTAs: for launches of so few queries that each warp's own chain of dependent
-// loads decides their time.
+// registers capped for 8 CTAs per SM (FP32 rows), 6 (filter) or 9 (exact codes, which
+// have this shape only: 2 x 500k SIFT-like rows S1 4.13 ms; 8 CTAs 4.24, 10 with spills
+// 4.41); 1 = the full rows in flight, 4 CTAs; 2 = a whole batch of rows in flight
+// (as far as 128 registers hold it), 2 CTAs: for launches of so few queries that each
+// warp's own chain of dependent loads decides their time.
 // A tuned variant number v selects shape v & 1 and, if v & 2, the L2
 // prefetch of the runner-up's neighbourhood during each expansion.
 constexpr int kLatencyShape = 2;
@@ -33,7 +29,6 @@ struct Variant {
                                     : MODE == kCodeFilter ? (VAR == 0 ? 6 : 4)
                                     : VAR == 0 ? 8 : 4;
 };
-constexpr int kVariants = 4;
 
 template <int F4, int MODE, int VAR>
 struct Layout {
@@ -68,7 +63,7 @@ struct CodeLayout {
 // both are full it replaces an entry of its home.  Forgetting an id costs its
 // re-evaluation if the search meets it again, never a result: an evaluated
 // vertex outside C is worse than the worst entry of C, and one inside C is
-// found there before it is inserted (kLossy below).
+// found there before it is inserted (`lossy`).
 //
 __device__ __forceinline__ int4 lds4(const int32_t *p) {
     int4 v;
