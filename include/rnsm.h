@@ -152,7 +152,7 @@ typedef struct {
 typedef struct {
     double wall_s;         /* rnsm_merge entry to return */
     double host_pivot_s;   /* host time in pivot selection */
-    int64_t ndc;           /* distance computations of all searches */
+    int64_t ndc;           /* vertices evaluated by all searches (by code or row) */
     int64_t expansions;    /* beam expansions of all searches */
     int64_t rechecks;      /* prune decisions re-decided in FP32 */
     int64_t pivots;        /* naive searches */
