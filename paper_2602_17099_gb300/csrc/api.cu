@@ -1311,6 +1311,7 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
         a.out_stride = p.k_plus;
         a.out_by_qidx = 1;
         a.stats = c.stats;
+        a.n_base = nmax;
         a.r_in = r_in_max;
         a.jobs = mb.jobs1;
         a.n_jobs = (int32_t)srcs.size();
@@ -1437,6 +1438,7 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
             a.out_stride = p.L;
             a.out_by_qidx = 1;
             a.stats = c.stats + 2;
+            a.n_base = nmax;
             a.r_in = r_in_max;
             a.jobs = mb.jobs4;
             a.n_jobs = (int32_t)(g1 - g0);
@@ -1458,6 +1460,7 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
             a.out_stride = p.L;
             a.out_by_qidx = 1;
             a.stats = c.stats + 4;
+            a.n_base = nmax;
             a.r_in = r_in_max;
             a.jobs = mb.jobs5;
             a.n_jobs = (int32_t)(g1 - g0);

@@ -95,7 +95,7 @@ struct SearchJob {
 // g selects the job and counts from the job's q_begin; nq is the total.
 struct SearchArgs {
     const float *base;      // searched vector set [n_base * dim]
-    int64_t n_base;
+    int64_t n_base;         // (jobs: at least the largest of theirs)
     const int32_t *adj;     // [n_base * r_in]
     int32_t r_in;           // (jobs: the largest of theirs)
     int32_t dim;

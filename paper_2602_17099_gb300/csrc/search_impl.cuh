@@ -4,6 +4,8 @@
 #pragma once
 #include <float.h>
 
+#include <algorithm>
+
 #include "internal.h"
 
 namespace rnsm {
@@ -57,6 +59,12 @@ struct CodeLayout {
     static_assert(W * G >= F4 && (W == 4 || F4 == W * G), "lanes cover a row");
 };
 
+// The visited table of a launch: 16-byte buckets, of ids (tag_shift 0) or of tags.
+struct TableShape {
+    uint32_t buckets;
+    int32_t shift, tag_shift;
+};
+
 // ---- the visited table ---------------------------------------------------
 // Ids in sets of two buckets of four (a bucket is one 16-byte shared load; -1
 // empty, slots filled in order): an id's home bucket, then its sibling, and if
@@ -64,7 +72,6 @@ struct CodeLayout {
 // re-evaluation if the search meets it again, never a result: an evaluated
 // vertex outside C is worse than the worst entry of C, and one inside C is
 // found there before it is inserted (`lossy`).
-//
 __device__ __forceinline__ int4 lds4(const int32_t *p) {
     int4 v;
     asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];"
@@ -96,6 +103,41 @@ __device__ __forceinline__ bool visit(int32_t *tab, uint32_t sets, int32_t id, b
                 bk ^= 1u;
             } else {
                 tab[4 * home + ((h >> 9) & 3u)] = id;
+                fresh = lost = true;
+                want = false;
+            }
+        }
+    }
+    lossy = lossy || __any_sync(0xffffffffu, lost);
+    return fresh;
+}
+
+// The same in half the memory, for beams over 64: a bucket of eight 16-bit tags is
+// a set.  With ids below 2^b, x = id * odd mod 2^b is a bijection, and x * sets =
+// set * 2^b + rest; within a set the rests are at least `sets` apart, so rest >>
+// log2(sets) tells its ids apart: as long as it has 15 bits (all ones is empty), tag and
+// set are the id.  shift = 32 - b; tag_shift = shift + log2(sets), rounded down.
+__device__ __forceinline__ bool visit_tags(int32_t *tab, uint32_t sets, int shift, int tag_shift, int32_t id, bool want,
+                                           bool &lossy) {
+    constexpr uint32_t kHigh = 0x80008000u;
+    const uint32_t x = ((uint32_t)id * 0x9E3779B1u) << shift;
+    const uint32_t set = __umulhi(x, sets), tag = (x * sets) >> tag_shift, both = tag * 0x10001u;
+    auto zero_half = [](uint32_t v) { return (v - 0x00010001u) & ~v & kHigh; };   // non-zero iff a half of v is zero
+    unsigned short *slots = reinterpret_cast<unsigned short *>(tab + 4 * set);
+    bool fresh = false, lost = false;
+    while (__any_sync(0xffffffffu, want)) {
+        if (want) {
+            const int4 w = lds4(tab + 4 * set);
+            const uint32_t a = (uint32_t)w.x, b = (uint32_t)w.y, c = (uint32_t)w.z, d = (uint32_t)w.w;
+            const int room = __popc((a & kHigh) >> 15 | (b & kHigh) >> 14 | (c & kHigh) >> 13 | (d & kHigh) >> 12);
+            if (zero_half(a ^ both) | zero_half(b ^ both) | zero_half(c ^ both) | zero_half(d ^ both)) {
+                want = false;
+            } else if (room > 0) {
+                const unsigned short old = atomicCAS(slots + 8 - room, (unsigned short)0xffffu, (unsigned short)tag);
+                fresh = old == 0xffffu;
+                want = !fresh && old != tag;   // another id took the slot: look again
+            } else {
+                slots[(x >> 9) & 7u] = (unsigned short)tag;
                 fresh = lost = true;
                 want = false;
             }
@@ -386,17 +428,17 @@ template <class T>
 __device__ __forceinline__ T fresh_read(const T &v) { return *const_cast<const volatile T *>(&v); }
 #define JF(f) (JOBS ? fresh_read(J->f) : a.f)
 
-// Shared memory: per warp the visited table (sets * 8 ids), then the batch's
+// Shared memory: per warp the visited table (16 bytes a bucket), then the batch's
 // new ids and those that pass the codes, scratch for C (and, for the ids that
 // pass, the query's row).
-__host__ __device__ constexpr size_t warp_smem_bytes(uint32_t sets, int efmax, int row_float4) {
-    return ((size_t)sets * 8 + 2 * kBatch) * sizeof(int32_t) + (size_t)efmax * sizeof(beam_t) +
+__host__ __device__ constexpr size_t warp_smem_bytes(uint32_t buckets, int efmax, int row_float4) {
+    return ((size_t)buckets * 4 + 2 * kBatch) * sizeof(int32_t) + (size_t)efmax * sizeof(beam_t) +
            (size_t)row_float4 * sizeof(float4);
 }
 
 template <int F4, int EFMAX, int MODE, int VAR, bool JOBS>
 __global__ void __launch_bounds__(kSearchWarps * 32, Variant<MODE, VAR>::kMinBlocks)
-search_kernel(const SearchArgs a, uint32_t sets, int prefetch) {
+search_kernel(const SearchArgs a, const TableShape table, int prefetch) {
     using Lay = Layout<F4, MODE, VAR>;
     using CLay = CodeLayout<F4, VAR>;
     constexpr int G = Lay::G, PER = EFMAX / 32;
@@ -404,8 +446,8 @@ search_kernel(const SearchArgs a, uint32_t sets, int prefetch) {
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     if (a.gate && (*a.gate & 3)) return;   // the inputs did not pass their checks
-    int32_t *tab = reinterpret_cast<int32_t *>(smem + (size_t)warp * warp_smem_bytes(sets, EFMAX, MODE == kCodeFilter ? F4 : 0));
-    int32_t *ci = tab + sets * 8;
+    int32_t *tab = reinterpret_cast<int32_t *>(smem + (size_t)warp * warp_smem_bytes(table.buckets, EFMAX, MODE == kCodeFilter ? F4 : 0));
+    int32_t *ci = tab + table.buckets * 4;
     int32_t *pass = ci + kBatch;
     beam_t *scratch = reinterpret_cast<beam_t *>(pass + kBatch);
     float4 *qrow_s = reinterpret_cast<float4 *>(scratch + EFMAX);
@@ -466,7 +508,7 @@ search_kernel(const SearchArgs a, uint32_t sets, int prefetch) {
 #pragma unroll
             for (int j = 0; j < CLay::W; ++j) qq = (int32_t)__dp4a(qc[j], qc[j], (uint32_t)qq);
         }
-        for (uint32_t i = lane; i < 2 * sets; i += 32) reinterpret_cast<int4 *>(tab)[i] = make_int4(-1, -1, -1, -1);
+        for (uint32_t i = lane; i < table.buckets; i += 32) reinterpret_cast<int4 *>(tab)[i] = make_int4(-1, -1, -1, -1);
         __syncwarp();
 
         beam_t k[PER];
@@ -542,7 +584,9 @@ search_kernel(const SearchArgs a, uint32_t sets, int prefetch) {
                     if (prefetch) pf = n0;
                 }
             }
-            const bool fresh = visit(tab, sets, cand, cand >= 0, lossy);
+            const bool fresh = EFMAX > 64 && table.tag_shift > 0
+                                   ? visit_tags(tab, table.buckets, table.shift, table.tag_shift, cand, cand >= 0, lossy)
+                                   : visit(tab, table.buckets / 2, cand, cand >= 0, lossy);
             const unsigned m = __ballot_sync(0xffffffffu, fresh);
             const int c = __popc(m);
             if (fresh) ci[__popc(m & lanemask_lt())] = cand;
@@ -607,24 +651,47 @@ search_kernel(const SearchArgs a, uint32_t sets, int prefetch) {
 
 #undef JF
 
-// Sets of the visited table.  A search meets up to 1.2 * ef * r_in different
+// The visited table of a launch.  A search meets up to 1.2 * ef * r_in different
 // vertices (DEEP-like rows, whose lists hardly overlap; SIFT-like ones half of
 // that); 1.25 * ef * r_in slots remember them all, and where that many would cost
 // resident warps, fewer: 1,536 slots against 4,096 took 24 % off the pivot searches
-// of 2 x 500k SIFT-like rows for 0.9 % more evaluations.
+// of 2 x 500k SIFT-like rows (ef 64) for 0.9 % more evaluations.  Beams over 64 take
+// tags, which remember twice as much in the same bytes: 24 a beam entry up to ef 128
+// and for lists over 48, else 20 (24 there cost warps: 10k DEEP-like queries, ef 256
+// 5.6 ms, 20 4.8).  Evaluations above those of an exact visited set (20k rows), and
+// time of 10k queries, with 1,536 or 2,048 ids and as below: DEEP-like R 32, ef 256
+// 20.9 -> 2.5 %, 5.1 -> 4.8 ms; embedding-like R 64, ef 128 15.5 -> 8.6 %, 8.9 -> 8.2 ms
+// and ef 256 40.4 -> 10.8 %, 20.5 -> 18.2 ms; 24 ids a beam entry: 0.6, 8.3 and 9.5 %, 7.8,
+// 9.4 and 45.5 ms.  (FP32 rows only, d = 128, ef 256: 6.2 -> 6.9 ms for 7 % fewer
+// evaluations.)  A tag costs some ten instructions more a lookup than an id, so short
+// lists keep ids (50k Gaussian rows, R 16, ef 128: 2,048 ids 1.13 ms, tags 1.22, 1,536 ids
+// 1.16); so do graphs whose ids need more than 15 bits beside the set.
 template <int VAR>
-uint32_t table_sets(int ef, int r_in) {
+TableShape table_shape(int ef, int r_in, int64_t n) {
     constexpr int kMost = VAR == kLatencyShape ? 8192 : VAR == 1 ? 2048 : 1536;
-    int e = ef * r_in + ef * r_in / 4;
-    if (e < 1024) e = 1024;
-    if (e > kMost) e = kMost;
-    return (uint32_t)(e + 63) / 64 * 8;
+    const int all = std::max(ef * r_in + ef * r_in / 4, 1024);
+    TableShape t = {};
+    if (VAR != kLatencyShape && ef > 64 && all > 2560) {
+        const int per = ef <= 128 || r_in > 48 ? 24 : 20;
+        const int buckets = (std::min(all, per * ef) + 63) / 64 * 8, lg = 31 - __builtin_clz((unsigned)buckets);
+        int b = lg + 1;
+        while (b < 31 && ((int64_t)1 << b) < n) ++b;
+        if (b - lg <= 15) {
+            t.buckets = (uint32_t)buckets;
+            t.shift = 32 - b;
+            t.tag_shift = 32 - b + lg;
+            return t;
+        }
+    }
+    const int slots = std::min(all, ef > 64 ? std::max(kMost, 2048) : kMost);
+    t.buckets = (uint32_t)(slots + 63) / 64 * 16;
+    return t;
 }
 
 template <int F4, int EFMAX, int MODE, int VAR, bool JOBS>
 cudaError_t launch_t(const SearchArgs &a, int prefetch, cudaStream_t st) {
-    const uint32_t sets = table_sets<VAR>(a.ef, a.r_in);
-    const size_t smem = (size_t)kSearchWarps * warp_smem_bytes(sets, EFMAX, MODE == kCodeFilter ? F4 : 0);
+    const TableShape table = table_shape<VAR>(a.ef, a.r_in, a.n_base);
+    const size_t smem = (size_t)kSearchWarps * warp_smem_bytes(table.buckets, EFMAX, MODE == kCodeFilter ? F4 : 0);
     auto kern = search_kernel<F4, EFMAX, MODE, VAR, JOBS>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
@@ -647,7 +714,7 @@ cudaError_t launch_t(const SearchArgs &a, int prefetch, cudaStream_t st) {
     int64_t want = (a.nq + kSearchWarps - 1) / kSearchWarps;
     int64_t grid = (int64_t)sms * per_sm;
     if (want < grid) grid = want < 1 ? 1 : want;
-    kern<<<(unsigned)grid, kSearchWarps * 32, smem, st>>>(a, sets, prefetch);
+    kern<<<(unsigned)grid, kSearchWarps * 32, smem, st>>>(a, table, prefetch);
     note_launches(1);
     return cudaGetLastError();
 }
