@@ -235,7 +235,8 @@ RNSM_API rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_
                        rnsm_stats *stats);
 
 /* Bytes of device workspace rnsm_merge takes for these inputs (without the
- * coded rows: a byte per component more). */
+ * coded rows: a byte per component more, and where there is room an eighth of that
+ * for the next larger call). */
 RNSM_API size_t rnsm_workspace_size(const rnsm_segment *segs, int32_t m, const rnsm_params *p);
 
 /* Frees the calling device's workspace (after synchronising). */

@@ -314,12 +314,15 @@ uint8_t *codes_acquire(size_t bytes, cudaStream_t st) {
         }
         w.ptr = nullptr;
         w.size = 0;
-        if (cudaMalloc(&w.ptr, bytes) != cudaSuccess) {
+        // room for an index that grows call by call; where there is none, what is needed
+        for (const size_t want : {bytes + (bytes >> 3), bytes}) {
+            if (cudaMalloc(&w.ptr, want) == cudaSuccess) {
+                w.size = want;
+                break;
+            }
             cudaGetLastError();
             w.ptr = nullptr;
-            return nullptr;
         }
-        w.size = bytes;
     }
     return static_cast<uint8_t *>(w.ptr);
 }

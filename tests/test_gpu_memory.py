@@ -1,0 +1,44 @@
+"""The device memory that the library keeps between calls: the coded rows' buffer
+beside the workspace."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rn():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_17099_gb300 import build as b
+    b.build()
+    from paper_2602_17099_gb300 import rnsm
+    return rnsm
+
+
+def _coded_search(rn, x, adj, nq):
+    # 16 * nq * 256 expected distances: coded rows if that is 8 a row
+    q = x[:nq]
+    seeds = torch.zeros((nq, 1), dtype=torch.int32, device="cuda")
+    return rn.search(x, adj, q, seeds, 256, 5)[0]
+
+
+def test_a_growing_index_does_not_reallocate_the_codes_each_call(rn):
+    # twelve calls, each with 3 % more rows (2.3 MB of codes and more, above the
+    # allocator's granularity of 2 MiB): growth by an eighth is four steps at most
+    top, d = 430_000, 256
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    x = torch.randn(top, d, generator=g, device="cuda")
+    adj = torch.randint(0, 300_000, (top, 2), generator=g, device="cuda", dtype=torch.int32)
+    _coded_search(rn, x[:300_000], adj[:300_000], 1300)
+    torch.cuda.synchronize()
+    free, changes = torch.cuda.mem_get_info()[0], 0
+    for i in range(1, 13):
+        n = int(300_000 * 1.03 ** i)
+        _coded_search(rn, x[:n], adj[:n], 1300)
+        now = torch.cuda.mem_get_info()[0]
+        changes += now != free
+        free = now
+    assert 1 <= changes <= 4
