@@ -27,6 +27,7 @@ def _coded_search(rn, x, adj, nq):
 def test_a_growing_index_does_not_reallocate_the_codes_each_call(rn):
     # twelve calls, each with 3 % more rows (2.3 MB of codes and more, above the
     # allocator's granularity of 2 MiB): growth by an eighth is four steps at most
+    rn.release_workspace()                 # (earlier calls may have left a larger buffer)
     top, d = 430_000, 256
     g = torch.Generator(device="cuda")
     g.manual_seed(1)
