@@ -10,8 +10,9 @@
  *   that the library grows on demand and keeps until rnsm_release_workspace()
  *   or process exit.  Calls that search dimensions of 64 and more also keep a
  *   byte per component of their rows (coded rows, kept and released alike; if
- *   there is no memory for them the FP32 rows are read alone), and so do the
- *   larger FP32 prunes of 64, 96 and 128 dimensions.
+ *   there is no memory for them the FP32 rows are read alone, and they are
+ *   given back when a workspace finds none), and so do the larger FP32 prunes
+ *   of 64, 96 and 128 dimensions.
  * - Vectors are row-major float32, rows contiguous, 16-byte aligned (dim must
  *   be a multiple of 4, at most 1024).  Calls that search (rnsm_search,
  *   rnsm_expand, rnsm_build_segment, rnsm_merge) need a dimension the search

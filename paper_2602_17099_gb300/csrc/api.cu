@@ -52,6 +52,7 @@ struct DevWs {
     void *ptr = nullptr;
     size_t size = 0;
 } g_ws[kMaxDev];
+DevWs g_codes[kMaxDev];   // coded rows: kept like the workspace, but a call can do without
 
 // The captured S4..S7 sequence of the last graph-mode call on a device.
 struct GraphCache {
@@ -101,6 +102,14 @@ rnsm_status ws_acquire(size_t bytes, Bump &b) {
         }
         size_t want = bytes + (bytes >> 3) + (1 << 20);
         cudaError_t e = cudaMalloc(&w.ptr, want);
+        if (e != cudaSuccess && g_codes[dev].ptr) {   // an earlier call's coded rows give way
+            cudaGetLastError();
+            CK(cudaDeviceSynchronize());
+            g_graphs[dev].reset();   // (captured launches may read them)
+            CK(cudaFree(g_codes[dev].ptr));
+            g_codes[dev] = DevWs();
+            e = cudaMalloc(&w.ptr, want);
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             w.ptr = nullptr;
@@ -289,8 +298,6 @@ rnsm_status check_segments(const rnsm_segment *segs, int32_t m, int32_t R) {
 //
 // A byte per dimension of every row of the call, in a grow-only buffer of its
 // own: unlike the workspace it may be missing (no memory: FP32 searches).
-
-DevWs g_codes[kMaxDev];
 
 struct Codes {
     uint8_t *rows = nullptr;   // coded rows by global id

@@ -43,3 +43,27 @@ def test_a_growing_index_does_not_reallocate_the_codes_each_call(rn):
         changes += now != free
         free = now
     assert 1 <= changes <= 4
+
+
+def test_kept_codes_give_way_to_the_workspace(rn):
+    # a search leaves 1 GB of codes behind; then the caller takes all memory but 256 MB,
+    # and a call needs a workspace of some 0.9 GB
+    n, d, m, kp = 4_000_000, 256, 20_000_000, 5
+    rn.release_workspace()
+    x = torch.zeros(n, d, device="cuda")
+    x[:, 0] = torch.arange(n, device="cuda") % 1000
+    adj = torch.randint(0, n, (n, 1), device="cuda", dtype=torch.int32)
+    nplus = torch.randint(0, m, (m, kp), device="cuda", dtype=torch.int32)
+    before = torch.cuda.mem_get_info()[0]
+    _coded_search(rn, x, adj, 8000)
+    assert before - torch.cuda.mem_get_info()[0] > n * d
+    outs = torch.empty(m * 14, dtype=torch.int32, device="cuda")   # room for the outputs
+    del outs
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - (256 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        offs, ids = rn.reverse_knn(nplus, kp)
+        assert int(offs[-1]) == m * kp and ids.shape[0] == m * kp
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+        rn.release_workspace()
