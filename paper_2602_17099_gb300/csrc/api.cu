@@ -302,6 +302,8 @@ rnsm_status check_segments(const rnsm_segment *segs, int32_t m, int32_t R) {
 struct Codes {
     uint8_t *rows = nullptr;   // coded rows by global id
     int32_t mode = kCodeNone;
+    // whether the prunes of source and of reverse-edge pools use them (filter mode)
+    int32_t source = 1, reverse = 1;
 };
 
 // RNSM_SEARCH_CODES: 0 FP32 rows only, 1 never by codes alone.
@@ -339,7 +341,8 @@ uint8_t *codes_acquire(size_t bytes, cudaStream_t st) {
 // valid after that check.  evals: distances that the call is expected to compute.  A row's code costs what some 8 evaluations gain (a pass
 // over 5 bytes a dimension against 3 gathered bytes and most of the arithmetic).
 rnsm_status code_table(const SegTable &t, int32_t dim, int32_t metric, int32_t checked, int64_t evals,
-                       const Ctl &c, cudaStream_t st, Codes &cd, CodeParams *params) {
+                       const Ctl &c, cudaStream_t st, Codes &cd, CodeParams *params,
+                       const CodeLists &lists = CodeLists()) {
     const int64_t n = t.off[t.m];
     cd = Codes();
     if (codes_dim_ok(dim) && codes_allowed() > 0 && evals >= 8 * n && n < INT32_MAX)
@@ -350,22 +353,50 @@ rnsm_status code_table(const SegTable &t, int32_t dim, int32_t metric, int32_t c
         return RNSM_OK;
     }
     CK(launch_code_scan(t, dim, checked, c.code_stats, c.err, st));
-    CK(launch_code_rows(t, dim, metric, cd.rows, c.code_stats, c.code_params, st));
+    CK(launch_code_rows(t, dim, cd.rows, c.code_stats, st));
+    CK(launch_code_params(t, dim, metric, lists, c.code_stats, c.code_params, st));
     CK(cudaMemcpyAsync(params, c.code_params, sizeof(CodeParams), cudaMemcpyDeviceToHost, st));
     return RNSM_OK;
 }
 
-// After the check: how the searches use the codes.
+// The lists that the prunes are sampled on: one table's rows of ids.
+CodeLists one_list(const int32_t *rows, int32_t len, float alpha, const int32_t *owners = nullptr,
+                   int64_t n_owners = 0) {
+    CodeLists l = {};
+    l.rows[0] = rows;
+    l.len[0] = rows ? len : 0;
+    l.alpha = alpha;
+    l.owners = owners;
+    l.n_owners = n_owners;
+    return l;
+}
+
+// Where the codes leave too many tests of a prune open, it does not use them: each
+// step of the walk with an open test waits for FP32 rows.  60k owners in clusters of
+// ever smaller radius, time over the FP32 kernel's by the share of sampled steps with
+// an open test: source pools (the FP32 walk) d = 64 0.84 at 0.41, 0.97 at 0.51, 1.14 at
+// 0.68; d = 96 0.85 at 0.45, 1.04 at 0.63; d = 128 0.87 at 0.39, 0.93 at 0.45, 1.04 at 0.52, 2.5
+// at 0.98; reverse-edge pools (the triangle) d = 64 0.92 at 0.42, 1.00 at 0.55; d = 96 1.00 at
+// 0.25, 0.98 at 0.38, 1.04 at 0.46; d = 128 0.89 at 0.08, 1.09 at 0.24.  DEEP-like rows 0.02 to 0.1.
+void code_prunes(Codes &cd, const CodeParams &p, int32_t dim) {
+    if (cd.mode != kCodeFilter) return;
+    const float share = p.steps > 0 ? (float)p.open_steps / (float)p.steps : 0.f;
+    cd.source = share <= (dim <= 96 ? 0.5f : 0.4f);
+    cd.reverse = share <= (dim <= 64 ? 0.5f : dim <= 96 ? 0.3f : 0.15f);
+}
+
+// After the check: how the searches and prunes use the codes.
 void code_mode(Codes &cd, const CodeParams &p, int32_t dim, int32_t metric) {
     cd.mode = kCodeNone;
     if (!cd.rows) return;
     if (p.exact && metric == RNSM_METRIC_L2 && dim <= 256 && codes_allowed() > 1) cd.mode = kCodeExact;
     else if (p.useful) cd.mode = kCodeFilter;
+    code_prunes(cd, p, dim);
 }
 
 // The codes for the prunes.
 void prune_codes(PruneArgs &a, const Codes &cd, const Ctl &c) {
-    if (cd.mode == kCodeNone) return;
+    if (cd.mode == kCodeNone || !(a.csr_offs ? cd.reverse : cd.source)) return;
     a.codes = cd.rows;
     a.code_params = cd.mode == kCodeExact ? nullptr : c.code_params;
 }
@@ -760,7 +791,9 @@ rnsm_status rnsm_prune(const float *vecs, int64_t n, int32_t dim, const int32_t 
     CodeParams code_params;
     const int64_t evals = prec == RNSM_PREC_FP32 && prune_code_ok(dim, metric) && w_len <= kPruneSmallMax ? nv * w_len : 0;
     const bool coding = evals >= 8 * n;
-    if (coding) TRY(code_table(one_table(vecs, n), dim, metric, 1, evals, c, st, codes, &code_params));
+    if (coding)
+        TRY(code_table(one_table(vecs, n), dim, metric, 1, evals, c, st, codes, &code_params,
+                       one_list(pool, w_len, alpha, owners, nv)));
     CK(launch_validate(coding ? nullptr : vecs, n * dim, {owners, nv, n, 0}, {pool, nv * w_len, n, -1}, {}, c.err, st));
     const bool gated = qprec == 0 && !coding && nv <= kGateOwners;   // FP32 kernels: one wait, at the end
     if (!gated) TRY(check_err_word(c, st));
@@ -819,7 +852,9 @@ rnsm_status rnsm_reverse_edges(const float *vecs, int64_t n, int32_t dim, int32_
     Codes codes;
     CodeParams code_params;
     const bool coding = prune_code_ok(dim, metric) && 16 * ne >= 8 * n;
-    if (coding) TRY(code_table(one_table(vecs, n), dim, metric, 1, 16 * ne, c, st, codes, &code_params));
+    if (coding)
+        TRY(code_table(one_table(vecs, n), dim, metric, 1, 16 * ne, c, st, codes, &code_params,
+                       one_list(lists, R, alpha)));
     CK(launch_validate(coding ? nullptr : vecs, n * dim, {lists, n * R, n, -1}, {eu, ne, n, 0}, {ev, ne, n, 0}, c.err,
                        st));
     TRY(check_err_word(c, st));
@@ -909,8 +944,19 @@ rnsm_status rnsm_build_segment(const float *vecs, int64_t n, int32_t dim, const 
         CK(launch_fill(out_adj, n * p.R, -1, st));
         CK(cudaStreamSynchronize(st));
     }
-    int64_t inserted = 1;
+    // the prunes are sampled again as the graph grows (a wait each)
+    const bool sampling = codes.mode == kCodeFilter && prune_code_ok(dim, p.metric);
+    int64_t inserted = 1, sample_at = 4096;
     while (inserted < n) {
+        if (sampling && inserted >= sample_at) {
+            CodeLists l = one_list(out_adj, p.R, p.alpha, order, inserted);
+            l.by_id = 1;
+            CK(launch_code_params(tab, dim, p.metric, l, c.code_stats, c.code_params, st));
+            CK(cudaMemcpyAsync(&code_params, c.code_params, sizeof(code_params), cudaMemcpyDeviceToHost, st));
+            CK(cudaStreamSynchronize(st));
+            code_prunes(codes, code_params, dim);
+            sample_at = 4 * inserted;
+        }
         int64_t bsz = inserted < B ? inserted : B;
         if (bsz > n - inserted) bsz = n - inserted;
         SearchArgs a = search_defaults();
@@ -1251,7 +1297,13 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
     for (const PlanEdge &e : pl) evals += search_evals(segs[e.src].n, cm ? p.L : p.ef_slide);
     if (!cm)
         for (int32_t s : srcs) evals += search_evals(segs[s].n, p.k_plus + 1);
-    TRY(code_table(tab, dim, p.metric, m, evals, c, st, codes, &code_params));
+    CodeLists lists = {};
+    lists.alpha = p.alpha;
+    for (int32_t s = 0; s < m; ++s) {
+        lists.rows[s] = segs[s].r_in > 0 ? segs[s].adj : nullptr;
+        lists.len[s] = segs[s].r_in;
+    }
+    TRY(code_table(tab, dim, p.metric, m, evals, c, st, codes, &code_params, lists));
     for (int32_t s = 0; s < m; ++s)
         if (segs[s].adj && segs[s].r_in > 0)
             CK(launch_validate_graph(segs[s].adj, segs[s].n, segs[s].r_in, c.err, st));
@@ -1596,7 +1648,8 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
         // graph mode: capture once, replay while the key matches
         std::string key = graph_key(segs, m, p, pl, out_adj, b.base, np, nf, dim, qprec);
         key.append(reinterpret_cast<const char *>(&codes.rows), sizeof(codes.rows));
-        key.append(reinterpret_cast<const char *>(&codes.mode), sizeof(codes.mode));
+        for (const int32_t v : {codes.mode, codes.source, codes.reverse})
+            key.append(reinterpret_cast<const char *>(&v), sizeof(v));
         GraphCache &gc = g_graphs[cur_device()];
         const bool replay = gc.exec && gc.key == key;
         if (!replay) {

@@ -40,11 +40,15 @@ long long launches_so_far();
 
 // Coded rows (codes.cu): a byte per dimension on one grid lo + s * c for all
 // the rows of a call.  CodeStats: what the passes over the rows gather (starts as zeros).
-// CodeParams: the searches' constants, read on the device.
+// CodeParams: the constants of the searches and prunes, read on the device.
+constexpr int kCodeSamples = 64;
 struct CodeStats {
     uint32_t omin_inv, omax;   // smallest (inverted) and largest component, order-preserving bits
     int32_t fraction;      // a component is no integer
     uint32_t err2, norm2;  // largest squared residual and squared row norm (float bits)
+    int32_t done;          // samples taken
+    int32_t steps, open_steps;   // as CodeParams
+    float pair_d2[kCodeSamples], pair_norm2[kCodeSamples];   // the sampled pairs: distance, sum of norms
 };
 struct CodeParams {
     float scale, inv_scale;  // s; 0: no codes
@@ -52,6 +56,19 @@ struct CodeParams {
     float norm2;             // largest squared row norm
     int32_t exact;           // integers, s = 1: code distances are the distances
     int32_t useful;          // err is small against the rows' distances
+    int32_t steps;           // sampled prunes: kept rows that later candidates are tested against,
+    int32_t open_steps;      // and those of them that a test is left open for by the codes
+};
+// The candidate lists that the prunes are sampled on: a row of ids (of their segment)
+// for each owner.  owners null: of every row, by segment; else of the listed ids (of
+// segment 0), in their order or (by_id) by id.
+struct CodeLists {
+    const int32_t *rows[kMaxSeg];   // null: none
+    int32_t len[kMaxSeg];
+    const int32_t *owners;
+    int64_t n_owners;
+    int32_t by_id;
+    float alpha;
 };
 enum CodeMode : int32_t { kCodeNone = 0, kCodeFilter = 1, kCodeExact = 2 };
 bool codes_dim_ok(int dim);
@@ -59,8 +76,9 @@ bool codes_dim_ok(int dim);
 // the statistics, in one pass over the table's rows; then the codes (rows by global id) and the constants.
 cudaError_t launch_code_scan(const SegTable &t, int32_t dim, int32_t checked, CodeStats *s, int32_t *err,
                              cudaStream_t st);
-cudaError_t launch_code_rows(const SegTable &t, int32_t dim, int32_t metric, uint8_t *codes, CodeStats *s,
-                             CodeParams *p, cudaStream_t st);
+cudaError_t launch_code_rows(const SegTable &t, int32_t dim, uint8_t *codes, CodeStats *s, cudaStream_t st);
+cudaError_t launch_code_params(const SegTable &t, int32_t dim, int32_t metric, const CodeLists &lists, CodeStats *s,
+                               CodeParams *p, cudaStream_t st);
 // Launches of up to this many queries take the search's latency shape, which
 // does not filter by codes.
 constexpr int64_t kLatencyQueries = 1216;

@@ -122,3 +122,29 @@ def test_a_tuned_choice_of_codes_does_not_outlive_them(rn, monkeypatch):
     second, st = rn.merge(segs, rn.params(16, 24, prec=1))
     assert 4 not in st["prune_kernel"]
     assert torch.equal(first, second)
+
+
+def _clusters(n, d, radius, seed):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    c = torch.nn.functional.normalize(torch.randn(n // 200, d, generator=g, device="cuda"), dim=1)
+    x = c[torch.randint(0, n // 200, (n,), generator=g, device="cuda")]
+    x = x + radius / d ** 0.5 * torch.randn(n, d, generator=g, device="cuda")
+    return torch.nn.functional.normalize(x, dim=1).contiguous()
+
+
+@pytest.mark.parametrize("d", [64, 96, 128])
+@pytest.mark.parametrize("radius,coded", [(3.0, True), (0.1, False)])
+def test_tight_clusters_are_pruned_over_fp32_rows(rn, monkeypatch, d, radius, coded):
+    # neighbours at 0.08 of the distance of rows far apart, the codes' bound at 0.02 of
+    # it: most steps of a prune leave a test open, so the codes serve the searches alone
+    X = _clusters(20_000, d, radius, d)
+    segs = [(x, *rn.build_segment(x, 32, 64)) for x in (X[:10_000].clone(), X[10_000:].clone())]
+    got, st = rn.merge(segs, rn.params(32, 64))
+    assert (st["prune_kernel"][0] == 4) == coded
+    assert (st["prune_kernel"][1] == 4) == coded
+    monkeypatch.setenv("RNSM_SEARCH_CODES", "0")
+    for x, adj, e in segs:
+        a, entry = rn.build_segment(x, 32, 64)
+        assert entry == e and torch.equal(a, adj)
+    assert torch.equal(rn.merge(segs, rn.params(32, 64))[0], got)
