@@ -225,10 +225,14 @@ rnsm_status ctl_reset(const Ctl &c, cudaStream_t st) {
     return RNSM_OK;
 }
 
-rnsm_status check_err_word(const Ctl &c, cudaStream_t st) {
-    int32_t err = 0;
-    CK(cudaMemcpyAsync(&err, c.err, sizeof(err), cudaMemcpyDeviceToHost, st));
+// Waits for the stream and reads the error word (and, in the same copy, the codes'
+// constants: a copy of their own to pageable memory would be a second wait).
+rnsm_status check_err_word(const Ctl &c, cudaStream_t st, CodeParams *params = nullptr) {
+    CtlBlock h;
+    CK(cudaMemcpyAsync(&h, c.err, params ? sizeof(h) : sizeof(h.err), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    const int32_t err = h.err;
+    if (params) *params = h.code_params;
     if (err & 1) return fail(RNSM_EGRAPH, "adjacency holds a vertex id outside [-1, n)");
     if (err & 2) return fail(RNSM_EGRAPH, "vectors hold a non-finite value");
     if (err & 16) return fail(RNSM_EGRAPH, "a prune pool exceeded 4096 candidates");
@@ -337,12 +341,13 @@ uint8_t *codes_acquire(size_t bytes, cudaStream_t st) {
 }
 
 // Validates the rows of the table's first `checked` segments (the error word is
-// read by the caller's check) and, where it pays, codes all of them; *params is
-// valid after that check.  evals: distances that the call is expected to compute.  A row's code costs what some 8 evaluations gain (a pass
-// over 5 bytes a dimension against 3 gathered bytes and most of the arithmetic).
+// read by the caller's check) and, where it pays, codes all of them; c.code_params is
+// valid after that check.  evals: distances that the call is expected to compute.  A
+// row's code costs what some 8 evaluations gain (a pass over 5 bytes a dimension
+// against 3 gathered bytes and most of the arithmetic).
 rnsm_status code_table(const SegTable &t, int32_t dim, int32_t metric, int32_t checked, int64_t evals,
-                       const Ctl &c, cudaStream_t st, Codes &cd, CodeParams *params,
-                       const CodeLists &lists = CodeLists()) {
+                       const Ctl &c, cudaStream_t st, Codes &cd,
+                       const CodeLists &lists = CodeLists(), bool exact_only = false) {
     const int64_t n = t.off[t.m];
     cd = Codes();
     if (codes_dim_ok(dim) && codes_allowed() > 0 && evals >= 8 * n && n < INT32_MAX)
@@ -352,12 +357,23 @@ rnsm_status code_table(const SegTable &t, int32_t dim, int32_t metric, int32_t c
             CK(launch_validate_vecs(t.base[s], (t.off[s + 1] - t.off[s]) * dim, c.err, st));
         return RNSM_OK;
     }
+    if (exact_only) CK(cudaMemsetAsync(&c.code_stats->exact_only, 1, sizeof(int32_t), st));
     CK(launch_code_scan(t, dim, checked, c.code_stats, c.err, st));
     CK(launch_code_rows(t, dim, cd.rows, c.code_stats, st));
     CK(launch_code_params(t, dim, metric, lists, c.code_stats, c.code_params, st));
-    CK(cudaMemcpyAsync(params, c.code_params, sizeof(CodeParams), cudaMemcpyDeviceToHost, st));
     return RNSM_OK;
 }
+
+// Prune calls of fewer owners, and reverse-edge calls of fewer lists, read FP32 rows:
+// codes cost four launches and a wait, and a warp an owner fills the chip late.  FP32
+// kernels and codes, us, d = 64 / 96 / 128.  Pools of 64, DEEP-like rows: 1,000 owners 106 /
+// 125 / 134 and 169 / 168 / 163, 2,000 132 / 149 / 163 and 160 / 158 / 165, 4,000 165 / 227 / 256
+// and 160 / 162 / 203; SIFT-like: 1,000 108 / 123 / 139 and 109 / 121 / 123, 2,000 123 / 143 / 153
+// and 116 / 119 / 121.  Back edges, 11 a list, DEEP-like rows: 4,000 lists 202 / 231 / 251 and
+// 372 / 372 / 372, 12,000 335 / 382 / 420 and 383 / 400 / 423, 16,000 432 / 455 / 521 and 428 / 427 /
+// 548; SIFT-like (exact codes pay earlier): 4,000 376 / 394 / 413 and 384 / 388 / 414, 8,000 558 /
+// 597 / 600 and 517 / 526 / 541.
+constexpr int64_t kCodePrune = 1536, kExactReverse = 6144, kCodeReverse = 14336;
 
 // The lists that the prunes are sampled on: one table's rows of ids.
 CodeLists one_list(const int32_t *rows, int32_t len, float alpha, const int32_t *owners = nullptr,
@@ -509,6 +525,7 @@ rnsm_status reverse_into(const SegTable &tab, int32_t dim, const rnsm_params &p,
     a.csr_offs = r.offs;
     a.csr_ids = r.ids;
     a.csr_max = csr_max;
+    a.csr_most = cap;
     a.out = lists;
     if (codes) prune_codes(a, *codes, c);
     a.err = c.err;
@@ -648,12 +665,12 @@ rnsm_status rnsm_search(const float *vecs, int64_t n, int32_t dim, const int32_t
     Codes codes;
     CodeParams code_params;
     const bool gated = nq <= kLatencyQueries;   // few queries: one wait, at the end
-    if (!gated) TRY(code_table(tab, dim, metric, 1, search_evals(nq, ef), c, st, codes, &code_params));
+    if (!gated) TRY(code_table(tab, dim, metric, 1, search_evals(nq, ef), c, st, codes));
     // adjacency and seeds: -1 or a vertex
     CK(launch_validate(gated ? vecs : nullptr, n * dim, {adj, adj ? n * r_in : 0, n, -1}, {seeds, nq * n_seeds, n, -1},
                        {}, c.err, st));
     if (!gated) {
-        TRY(check_err_word(c, st));
+        TRY(check_err_word(c, st, &code_params));
         code_mode(codes, code_params, dim, metric);
     }
     SearchArgs a = search_defaults();
@@ -703,9 +720,9 @@ rnsm_status rnsm_expand(const float *vecs, int64_t n, int32_t dim, const int32_t
     TRY(ctl_reset(c, st));
     Codes codes;
     CodeParams code_params;
-    TRY(code_table(one_table(vecs, n), dim, metric, 1, search_evals(n, k_plus + 1), c, st, codes, &code_params));
+    TRY(code_table(one_table(vecs, n), dim, metric, 1, search_evals(n, k_plus + 1), c, st, codes));
     if (adj && r_in > 0) CK(launch_validate_graph(adj, n, r_in, c.err, st));
-    TRY(check_err_word(c, st));
+    TRY(check_err_word(c, st, &code_params));
     code_mode(codes, code_params, dim, metric);
     SearchArgs a = search_defaults();
     a.code_mode = codes.mode;
@@ -790,13 +807,13 @@ rnsm_status rnsm_prune(const float *vecs, int64_t n, int32_t dim, const int32_t 
     Codes codes;
     CodeParams code_params;
     const int64_t evals = prec == RNSM_PREC_FP32 && prune_code_ok(dim, metric) && w_len <= kPruneSmallMax ? nv * w_len : 0;
-    const bool coding = evals >= 8 * n;
+    const bool coding = evals >= 8 * n && nv >= kCodePrune;
     if (coding)
-        TRY(code_table(one_table(vecs, n), dim, metric, 1, evals, c, st, codes, &code_params,
+        TRY(code_table(one_table(vecs, n), dim, metric, 1, evals, c, st, codes,
                        one_list(pool, w_len, alpha, owners, nv)));
     CK(launch_validate(coding ? nullptr : vecs, n * dim, {owners, nv, n, 0}, {pool, nv * w_len, n, -1}, {}, c.err, st));
     const bool gated = qprec == 0 && !coding && nv <= kGateOwners;   // FP32 kernels: one wait, at the end
-    if (!gated) TRY(check_err_word(c, st));
+    if (!gated) TRY(check_err_word(c, st, &code_params));
     if (coding) code_mode(codes, code_params, dim, metric);
     SegTable tab;
     std::memset(&tab, 0, sizeof(tab));
@@ -851,13 +868,13 @@ rnsm_status rnsm_reverse_edges(const float *vecs, int64_t n, int32_t dim, int32_
     TRY(ctl_reset(c, st));
     Codes codes;
     CodeParams code_params;
-    const bool coding = prune_code_ok(dim, metric) && 16 * ne >= 8 * n;
+    const bool coding = prune_code_ok(dim, metric) && 16 * ne >= 8 * n && n >= kExactReverse;
     if (coding)
-        TRY(code_table(one_table(vecs, n), dim, metric, 1, 16 * ne, c, st, codes, &code_params,
-                       one_list(lists, R, alpha)));
+        TRY(code_table(one_table(vecs, n), dim, metric, 1, 16 * ne, c, st, codes,
+                       one_list(lists, R, alpha), n < kCodeReverse));
     CK(launch_validate(coding ? nullptr : vecs, n * dim, {lists, n * R, n, -1}, {eu, ne, n, 0}, {ev, ne, n, 0}, c.err,
                        st));
-    TRY(check_err_word(c, st));
+    TRY(check_err_word(c, st, &code_params));
     if (coding) code_mode(codes, code_params, dim, metric);
     SegTable tab;
     std::memset(&tab, 0, sizeof(tab));
@@ -931,8 +948,8 @@ rnsm_status rnsm_build_segment(const float *vecs, int64_t n, int32_t dim, const 
     const SegTable tab = one_table(vecs, n);
     Codes codes;
     CodeParams code_params;
-    TRY(code_table(tab, dim, p.metric, 1, search_evals(n, p.L), c, st, codes, &code_params));
-    TRY(check_err_word(c, st));
+    TRY(code_table(tab, dim, p.metric, 1, search_evals(n, p.L), c, st, codes));
+    TRY(check_err_word(c, st, &code_params));
     code_mode(codes, code_params, dim, p.metric);
     {
         std::vector<int32_t> h((size_t)n);
@@ -1303,11 +1320,11 @@ rnsm_status rnsm_merge(const rnsm_segment *segs, int32_t m, const rnsm_params *p
         lists.rows[s] = segs[s].r_in > 0 ? segs[s].adj : nullptr;
         lists.len[s] = segs[s].r_in;
     }
-    TRY(code_table(tab, dim, p.metric, m, evals, c, st, codes, &code_params, lists));
+    TRY(code_table(tab, dim, p.metric, m, evals, c, st, codes, lists));
     for (int32_t s = 0; s < m; ++s)
         if (segs[s].adj && segs[s].r_in > 0)
             CK(launch_validate_graph(segs[s].adj, segs[s].n, segs[s].r_in, c.err, st));
-    TRY(check_err_word(c, st));
+    TRY(check_err_word(c, st, &code_params));
     code_mode(codes, code_params, dim, p.metric);
     auto use_codes = [&](SearchArgs &a) {
         a.code_mode = codes.mode;

@@ -75,13 +75,15 @@ __global__ void __launch_bounds__(256) code_scan_kernel(const SegTable t, int di
 }
 
 // lo and s of the scanned rows; s = 0: no codes (a range that is empty, not
-// finite, or so large or small that the bounds below could leave FP32's range).
+// finite, or so large or small that the bounds below could leave FP32's range;
+// or only exact codes are wanted).
 __device__ __forceinline__ void code_grid(const CodeStats *st, float &lo, float &s) {
     const float a = order_value(~st->omin_inv), b = order_value(st->omax);
     const float range = b - a;
     lo = a;
     s = 0.f;
     if (!st->fraction && range <= 255.f && fabsf(a) <= 65536.f) s = 1.f;
+    else if (st->exact_only) s = 0.f;
     else if (range > 1e-12f && range < 1e12f && fabsf(a) < 1e12f) s = range / 255.f;
 }
 

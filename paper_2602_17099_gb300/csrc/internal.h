@@ -45,6 +45,7 @@ constexpr int kCodeSamples = 64;
 struct CodeStats {
     uint32_t omin_inv, omax;   // smallest (inverted) and largest component, order-preserving bits
     int32_t fraction;      // a component is no integer
+    int32_t exact_only;    // set before the scan: no codes but exact ones
     uint32_t err2, norm2;  // largest squared residual and squared row norm (float bits)
     int32_t done;          // samples taken
     int32_t steps, open_steps;   // as CodeParams
@@ -183,6 +184,7 @@ struct PruneArgs {
     const int64_t *csr_offs;
     const int32_t *csr_ids;
     int32_t csr_max;          // longest CSR row (sizes the pool buffer)
+    int64_t csr_most;         // at most this many CSR entries in all
     int32_t *out;             // rows by owner gid (out_by_index: by i), stride R
     int32_t out_by_index;
     int32_t emit_lo, emit_hi; // kept ids in [emit_lo, emit_hi) emit (u, owner)

@@ -62,6 +62,7 @@ cudaError_t run_variant(const PruneArgs &a, int var, cudaStream_t st) {
 }
 
 constexpr int64_t kCodeFirst = 16384;
+constexpr int64_t kCodeReverseFirst = 7168;
 
 // The variants that apply to a call, the default (the first) included.
 int variants_of(const PruneArgs &a, int *out) {
@@ -72,7 +73,15 @@ int variants_of(const PruneArgs &a, int *out) {
     // ms; the FP32 walk 2.82).  With tiles asked for they come first from kCodeFirst owners
     // on (300k DEEP-like rows in 6 plan edges, S6 + S7: 8.0 ms, the BF16 pair tile 11.8);
     // below that the launch is short either way and the tiles stay the default.
-    const bool code_ok = a.codes && prune_code_ok(a.dim, a.metric) && a.lenA + a.lenB <= kPruneSmallMax;
+    // Reverse-edge pools of fewer lists (with entries) stay with the triangle unless the
+    // codes are exact: its five warps an owner finish a small launch sooner than one.  S7 of
+    // 2 x n DEEP-like rows, d = 64 / 96 / 128, triangle and coded walk: n = 4,000 0.17 / 0.16 /
+    // 0.18 and 0.25 / 0.20 / 0.21 ms; 6,000 0.18 / 0.19 / 0.20 and 0.22 / 0.21 / 0.21; 8,000 0.21 /
+    // 0.23 / 0.26 and 0.23 / 0.21 / 0.22.  Graph builds of 4,000 rows (rounds of 64): 17.0 / 17.3 /
+    // 18.2 and 21.7 / 21.1 / 21.0 ms.
+    const bool small_reverse =
+        a.csr_offs && a.code_params && (a.n_owners < kCodeReverseFirst || a.csr_most < kCodeReverseFirst);
+    const bool code_ok = a.codes && prune_code_ok(a.dim, a.metric) && a.lenA + a.lenB <= kPruneSmallMax && !small_reverse;
     const bool code_first = code_ok && (a.prec == 0 || a.n_owners >= kCodeFirst);
     if (code_first) out[n++] = kVarCode;
     if (code_first && a.prec == 0 && forced_prune_variant() < 0) return n;

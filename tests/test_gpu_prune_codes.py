@@ -148,3 +148,61 @@ def test_tight_clusters_are_pruned_over_fp32_rows(rn, monkeypatch, d, radius, co
         a, entry = rn.build_segment(x, 32, 64)
         assert entry == e and torch.equal(a, adj)
     assert torch.equal(rn.merge(segs, rn.params(32, 64))[0], got)
+
+
+@pytest.mark.parametrize("d", [64, 96, 128])
+def test_small_reverse_edge_pools_of_real_rows_take_the_triangle(rn, monkeypatch, d):
+    rng = np.random.default_rng(d)
+    for kind, n, want in (("wide", 2000, [4, 0]), ("integers", 2000, [4, 4]), ("wide", 8000, [4, 4])):
+        X = torch.from_numpy(_rows(2 * n, d, rng)).cuda() if kind == "integers" else _clusters(2 * n, d, 3.0, n)
+        segs = [(x, *rn.build_segment(x, 16, 32)) for x in (X[:n].clone(), X[n:].clone())]
+        got, st = rn.merge(segs, rn.params(16, 32))
+        assert st["prune_kernel"] == want
+        monkeypatch.setenv("RNSM_SEARCH_CODES", "0")
+        assert torch.equal(rn.merge(segs, rn.params(16, 32))[0], got)
+        monkeypatch.delenv("RNSM_SEARCH_CODES")
+
+
+def _kernels(f):
+    """The names of the kernels that a call launches ("" where they cannot be traced)."""
+    from torch.profiler import ProfilerActivity, profile
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        f()
+        torch.cuda.synchronize()
+    return " ".join(e.key for e in prof.key_averages())
+
+
+# prune calls: distances enough for the rows to be coded (8 a row) from one candidate an
+# owner on; reverse edges: on both sides of the list counts from which integers and real
+# rows are coded
+@pytest.mark.parametrize("d", [64, 96, 128])
+@pytest.mark.parametrize("kind", ["integers", "wide"])
+def test_coded_calls_run_the_coded_kernel_and_equal_fp32(rn, monkeypatch, kind, d):
+    rng = np.random.default_rng(d)
+    make = lambda k: torch.from_numpy(_rows(k, d, rng)).cuda() if kind == "integers" else _clusters(k, d, 3.0, k)
+    n = 2000
+    X = make(n)
+    lists = rn.build_segment(X, 32, 64)[0]
+    two = torch.cat([lists, lists[lists[:, 0].long().clamp_min(0)]], 1)
+    calls = []
+    for w, nv in ((1, 8 * n), (2, 8 * n), (33, n), (64, 1536), (64, 1535)):
+        owners = torch.from_numpy(rng.integers(0, n, nv)).cuda()
+        pool = two[owners, :w].contiguous()
+        owners = owners.int()
+        calls.append((nv >= 1536, lambda o=owners, p=pool: rn.prune(X, o, p, 16, 1.2)))
+    for m in (6143, 6144, 14_335, 14_336):
+        Y = make(m)
+        adj = rn.build_segment(Y, 32, 64)[0]
+        v = torch.arange(m, device="cuda").repeat_interleave(12)
+        j = torch.from_numpy(rng.integers(0, 32, (2, len(v)))).cuda()
+        u = adj[adj[v, j[0]].long().clamp_min(0), j[1]]
+        eu, ev = u[u >= 0].contiguous(), v[u >= 0].int()
+        coded = m >= (6144 if kind == "integers" else 14_336)
+        calls.append((coded, lambda y=Y, l=adj, a=eu, b=ev: rn.reverse_edges(y, l.clone(), a, b, 1.2)))
+    for coded, call in calls:
+        monkeypatch.delenv("RNSM_SEARCH_CODES", raising=False)
+        got, names = call(), _kernels(call)
+        if names:
+            assert ("prune_code_kernel" in names) == coded
+        monkeypatch.setenv("RNSM_SEARCH_CODES", "0")
+        assert torch.equal(call(), got)
