@@ -39,10 +39,8 @@ from workloads import generators as gen  # noqa: E402
 METRIC = "merged_vertices_per_s"
 UNIT = "vertices/s"
 SEARCH_SRC = [os.path.join(ROOT, "paper_2602_17099_gb300", "csrc", f)
-              for f in ("search_impl.cuh", "search.cu", "codes.cu")]
+              for f in ("search_impl.cuh", "search.cu", "codes.cu", "common.cuh")]
 PROFILE = os.path.join(ROOT, "profiles", "search_kernel_sift2x500k.txt")
-PRUNE_SRC = [os.path.join(ROOT, "paper_2602_17099_gb300", "csrc", f)
-             for f in ("prune.cu", "common.cuh")]
 L2_PROFILE = os.path.join(ROOT, "profiles", "search_kernel_s5_sift2x200k.md")
 # the FP32 prune kernels of pools <= 64, by the variant number the library
 # reports (stats prune_kernel): their kernel name and committed ncu summaries
@@ -53,6 +51,14 @@ PRUNE_KERNELS = {
     4: ("prune_code_kernel", "prune_code_kernel_sift2x500k.txt", "prune_code_kernel_sift2x200k.md"),
 }
 PRUNE_DEFAULT_VARIANT = 4   # integer rows
+
+
+def prune_sources(variant=PRUNE_DEFAULT_VARIANT):
+    """The sources whose hash a capture of a prune kernel carries."""
+    return [os.path.join(ROOT, "paper_2602_17099_gb300", "csrc", f)
+            for f in ("prune_code.cu" if variant == 4 else "prune.cu", "common.cuh")]
+
+
 L2_METRIC, IP_METRIC = 0, 1
 
 
@@ -382,7 +388,7 @@ def _prune_profile(variant, k):
 
 def prune_profile_traffic(variant=PRUNE_DEFAULT_VARIANT):
     path = _prune_profile(variant, 1)
-    return path and profile_traffic(path, PRUNE_SRC, "prune sources sha256[:16]",
+    return path and profile_traffic(path, prune_sources(variant), "prune sources sha256[:16]",
                                     "dram bytes per S6 launch")
 
 
@@ -390,8 +396,22 @@ def prune_profile_fma(variant=PRUNE_DEFAULT_VARIANT):
     """FMA-pipe activity (percent of peak) of an FP32 small-pool prune kernel,
     from the committed small-case ncu capture of the current sources."""
     path = _prune_profile(variant, 2)
-    return path and profile_traffic(path, PRUNE_SRC, "prune sources sha256[:16]",
+    return path and profile_traffic(path, prune_sources(variant), "prune sources sha256[:16]",
                                     "fma pipe active pct (S6)")
+
+
+def row_codes(rows, dim, metric):
+    """How the library reads these workloads' rows: "exact" (integers spanning at most
+    255 at L2: a byte per component is the row), "filter" (a byte per component first,
+    FP32 rows of what it leaves open) or "none" (FP32 rows)."""
+    if dim not in (64, 96, 128, 256, 768):
+        return "none"
+    if metric == L2_METRIC and dim <= 256:
+        lo = min(float(r.min()) for r in rows)
+        hi = max(float(r.max()) for r in rows)
+        if hi - lo <= 255.0 and all(bool((r == r.round()).all()) for r in rows):
+            return "exact"
+    return "filter"
 
 
 def search_profile_l2():
@@ -582,8 +602,10 @@ def run_ours(args, ws, rank, local):
     s_bytes = s_ms = 0.0
     launches = 0
     n_search_launches = 0
-    # integer rows are read as codes, a byte per component (S6 says whether they were)
-    elt = 1 if stats[-1]["prune_kernel"][0] == 4 else 4
+    # coded rows: a byte per component (a filter's FP32 rows of what passes come on top
+    # and are not counted)
+    codes = row_codes(vd, W.dim, W.metric)
+    elt = 4 if codes == "none" else 1
     for st in stats:
         for i, ph in ((0, 1), (1, 4), (2, 5)):
             s_bytes += (st["search_ndc"][i] * W.dim * elt + st["search_exp"][i] * W.R * 4 +
@@ -610,18 +632,22 @@ def run_ours(args, ws, rank, local):
                    "algorithmic_bytes_per_launch": s_bytes / n_search_launches,
                    "avg_launch_ms": s_ms / n_search_launches,
                    "l2": search_profile_l2(),
-                   "bytes_per_component": elt,
-                   "note": "algorithmic bytes; most are served from L2 (see traffic and l2)"}
+                   "bytes_per_component": elt, "row_codes": codes,
+                   "note": "algorithmic bytes; most are served from L2 (see traffic and l2)" + (
+                       "; FP32 rows that pass the codes not counted" if codes == "filter" else "")}
     # roofline of the S6 source prune, in the unit of its per-owner gather: the
-    # owner row and its c = R + c_cross raw pool rows, d x 4 bytes each (coded: d), per
+    # owner row and its c = R + c_cross raw pool rows, d x 4 bytes each (the coded walk: d
+    # where the codes are the rows, else d x 5, codes and FP32 owner distances), per
     # owner (every source vertex), against the measured HBM copy bandwidth
     pool = W.R + (W.L + 1) // 2
-    b_per_owner = (pool + 1) * W.dim * elt
+    s6_var = stats[-1]["prune_kernel"][0]
+    s6_coded = codes if s6_var == 4 else "none"
+    b_per_owner = {"exact": (pool + 1) * W.dim, "filter": pool * W.dim * 5 + W.dim * 4,
+                   "none": (pool + 1) * W.dim * 4}[s6_coded]
     owners = sum(st["pivots"] + st["followers"] for st in stats)
     p_ms = sum(st["phase_ms"][6] for st in stats)
     n_p6 = len(stats) * (len(plan_used) if plan_used else 1)
     p_ach = owners * b_per_owner / (p_ms / 1000.0) / 1e9
-    s6_var = stats[-1]["prune_kernel"][0]
     s6_name = (PRUNE_KERNELS[s6_var][0] if pool <= 64 and s6_var in PRUNE_KERNELS
                else "prune_kernel")
     prune_roof = {"bound": "hbm",
@@ -633,19 +659,21 @@ def run_ours(args, ws, rank, local):
                   "algorithmic_bytes_per_owner": b_per_owner,
                   "avg_launch_ms": p_ms / n_p6}
     # the same launches as FP32 arithmetic: at most R x c occlusion tests per
-    # owner (the walk tests a candidate only against kept ones), 2 FLOP per
-    # dimension, against SMs x 128 FP32 lanes x 2 FLOP x the maximum SM clock
+    # owner (the walk tests a candidate only against kept ones; over codes in a filter
+    # only the c owner distances are FP32, but for the few tests it leaves open), 2 FLOP
+    # per dimension, against SMs x 128 FP32 lanes x 2 FLOP x the maximum SM clock
     sm_count = torch.cuda.get_device_properties(0).multi_processor_count
     alu_peak = sm_count * 128 * 2 * float(peaks.get("sm_max_mhz", 2070.0)) * 1e6 / 1e12
-    f_ach = owners * W.R * pool * W.dim * 2 / (p_ms / 1000.0) / 1e12
+    flop_per_owner = (1 if s6_coded == "filter" else W.R) * pool * W.dim * 2
+    f_ach = owners * flop_per_owner / (p_ms / 1000.0) / 1e12
     prune_flop = {"bound": "alu", "kernel": prune_roof["kernel"], "achieved_at_most": f_ach,
                   "peak": alu_peak, "unit": "TFLOP/s", "frac_at_most": f_ach / alu_peak,
                   "peak_source": "derived: %d SMs x 128 FP32 lanes x 2 FLOP x %.0f MHz" % (
                       sm_count, float(peaks.get("sm_max_mhz", 2070.0))),
-                  "flop_per_owner_at_most": W.R * pool * W.dim * 2,
+                  "flop_per_owner_at_most": flop_per_owner,
                   # measured: the FMA pipe's activity in the committed ncu capture
                   "fma_pipe_active_pct_ncu": prune_profile_fma(s6_var) if W.name == "sift2x500k" else None}
-    if s6_var == 4:   # integer dot products of coded rows: no FP32 arithmetic to rate
+    if s6_coded == "exact":   # integer dot products of coded rows: no FP32 arithmetic to rate
         prune_flop = None
     # the dominant kernel family of the FP32 step by live time goes first
     s7_ms = sum(st["phase_ms"][7] for st in stats)
