@@ -173,12 +173,14 @@ typedef struct {
      * on the owner distances of every 64th owner: [0] max |d~ - d64| / d64
      * (tile vs FP64), [1] max |d32 - d64| / d64 (the FP32 distance vs FP64),
      * [2] max |d~ - d32| / B (the share of its error bound B the tile used),
-     * [3] number of distances sampled.  Zero in FP32 mode and where no tile ran
-     * (prune_kernel: larger calls may take another variant). */
+     * [3] number of distances sampled.  Zero in FP32 mode and where no tile ran:
+     * with coded rows (L2, d = 64, 96, 128) prunes of 16,384 owners and more
+     * take those first, and the autotuner may choose them (prune_kernel 4). */
     double tile_error[4];
     /* BF16 / FP8 modes: occlusion tests the tensor-core tiles evaluated (the
      * share that was re-decided is rechecks / tile_tests, owner-distance
-     * re-decisions of the general tile included in rechecks).  Zero in FP32. */
+     * re-decisions of the general tile included in rechecks).  Zero where no
+     * tile ran, as above. */
     int64_t tile_tests;
     /* The prune kernel that served the last S6 call and the last S7 pool prune
      * (the autotuner's choice): 0 the FP32 register-blocked triangle, 1 the
@@ -302,7 +304,9 @@ RNSM_API rnsm_status rnsm_select_pivots(int64_t n, const int64_t *offs, const in
  *   nplus, k_plus, k   device N+ [n * k_plus]; N_k = its first k columns
  *   offs, ids          device CSR of R_k built from the same N_k
  *   pivot_of           device [n]: pivot of each follower, -1 for pivots
- *   n_pivots, rounds   host outputs (rounds may be NULL)
+ *   n_pivots, rounds   host outputs (rounds may be NULL); rounds: the parallel
+ *                      rounds, rounded up to a multiple of four (as the first
+ *                      version counted them, which looked after every fourth)
  */
 RNSM_API rnsm_status rnsm_select_pivots_gpu(const int32_t *nplus, int64_t n, int32_t k_plus,
                                             int32_t k, const int64_t *offs, const int32_t *ids,

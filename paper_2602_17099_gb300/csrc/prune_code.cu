@@ -1,5 +1,7 @@
 // The occlusion prune over coded rows (codes.cu): L2, d = 64, 96 or 128, pools of at
-// most 64 raw candidates, in FP32 mode.
+// most 64 raw candidates; in FP32 mode, and in the tile modes too from the owner count
+// that prune_route.cu gives.  Where sampled lists show that the codes would leave many
+// tests open (rows in tight clusters) the call does not use them (api.cu, code_prunes).
 //
 // What bounds the FP32 walk (prune.cu) is that a row of 128 floats a thread leaves
 // twelve warps per SM, each waiting on shared memory and barriers.  A coded row is
@@ -220,10 +222,10 @@ __global__ void __launch_bounds__(kCodeWarps * 32, code_blocks<W, kExact>())
                 s.order[lane] = ~0ull;
                 s.order[lane + 32] = ~0ull;
             } else {
-            K[0] = (id[0] >= 0 ? ((unsigned long long)(nv + n0 - 2u * v0) << 37) | ((unsigned long long)(uint32_t)id[0] << 6)
-                               : ~63ull) | (unsigned)lane;
-            K[1] = (id[1] >= 0 ? ((unsigned long long)(nv + n1 - 2u * v1) << 37) | ((unsigned long long)(uint32_t)id[1] << 6)
-                               : ~63ull) | (unsigned)(lane + 32);
+                K[0] = (id[0] >= 0 ? ((unsigned long long)(nv + n0 - 2u * v0) << 37) | ((unsigned long long)(uint32_t)id[0] << 6)
+                                   : ~63ull) | (unsigned)lane;
+                K[1] = (id[1] >= 0 ? ((unsigned long long)(nv + n1 - 2u * v1) << 37) | ((unsigned long long)(uint32_t)id[1] << 6)
+                                   : ~63ull) | (unsigned)(lane + 32);
             }
             s.key[lane] = K[0];
             s.key[lane + 32] = K[1];

@@ -61,6 +61,11 @@ cudaError_t run_variant(const PruneArgs &a, int var, cudaStream_t st) {
     return launch_prune_general(b, a.ovf_list, a.ovf_count, st);
 }
 
+// Not a crossing: S6 + S7 of 2 x n DEEP-like rows, BF16 pair tile and coded walk, d = 64 / 96 /
+// 128: n = 4,000 0.32 / 0.35 / 0.42 and 0.33 / 0.28 / 0.34 ms; 8,000 0.40 / 0.45 / 0.51 and 0.37 /
+// 0.37 / 0.40; 16,000 0.53 / 0.72 / 0.81 and 0.44 / 0.47 / 0.62; 24,000 0.74 / 0.90 / 1.02 and 0.51 /
+// 0.66 / 0.76.  Below it the tiles that the caller asked for run, and report their error
+// and tests (rnsm_stats); from it on some 0.2 ms a launch are worth more than that.
 constexpr int64_t kCodeFirst = 16384;
 constexpr int64_t kCodeReverseFirst = 7168;
 
@@ -71,8 +76,7 @@ int variants_of(const PruneArgs &a, int *out) {
     // so in FP32 mode nothing else is tried (2 x 500k SIFT-like rows, S6 + S7: 4.8 ms; the
     // FP32 walk 23.0, the BF16 pair tile 12.5, the FP8 one 14.7.  100k DEEP-like owners: 1.16
     // ms; the FP32 walk 2.82).  With tiles asked for they come first from kCodeFirst owners
-    // on (300k DEEP-like rows in 6 plan edges, S6 + S7: 8.0 ms, the BF16 pair tile 11.8);
-    // below that the launch is short either way and the tiles stay the default.
+    // on (300k DEEP-like rows in 6 plan edges, S6 + S7: 8.0 ms, the BF16 pair tile 11.8).
     // Reverse-edge pools of fewer lists (with entries) stay with the triangle unless the
     // codes are exact: its five warps an owner finish a small launch sooner than one.  S7 of
     // 2 x n DEEP-like rows, d = 64 / 96 / 128, triangle and coded walk: n = 4,000 0.17 / 0.16 /

@@ -89,7 +89,12 @@ int forced_variant() {
 // lane's share of a row is six float4 and few rows are in flight otherwise.
 // Embedding-like rows (768, filtered): S4 10.5 -> 5.6 ms, S5 15.0 -> 10.1 ms on
 // 3 x 20k; DEEP-like rows (96, FP32 only): S4 6.7 -> 5.4, S5 9.4 -> 9.1 ms on
-// 300k; SIFT-like rows (128, FP32 only) S5 8.6 -> 11.6 ms on 2 x 500k.
+// 300k; SIFT-like rows (128, FP32 only) S5 8.6 -> 11.6 ms on 2 x 500k.  The dimensions
+// with no merge behind them, 20k queries, ef 32 / 64 / 128, shape 0 and 1: 64 filtered 0.93 /
+// 1.49 / 2.96 and 1.11 / 1.82 / 3.50 ms, FP32 only 0.95 / 1.59 / 3.22 and 0.91 / 1.50 / 3.27;
+// 256 filtered 1.97 / 3.31 / 6.76 and 2.06 / 3.60 / 6.49, FP32 only 2.94 / 4.95 / 8.76 and 2.91 /
+// 4.85 / 9.10.  (Filtered against FP32 only: 64 0.92 / 1.49 / 2.95 and 0.91 / 1.52 / 3.14 ms, 128
+// 1.38 / 2.33 / 4.25 and 1.86 / 3.14 / 5.66.)
 int default_variant(int dim, int code_mode) {
     return dim == 768 || (dim == 96 && code_mode == kCodeNone) ? 1 : 0;
 }
