@@ -584,7 +584,7 @@ search_kernel(const SearchArgs a, const TableShape table, int prefetch) {
                     if (prefetch) pf = n0;
                 }
             }
-            const bool fresh = EFMAX > 64 && table.tag_shift > 0
+            const bool fresh = EFMAX > 64 && VAR != kLatencyShape && table.tag_shift > 0
                                    ? visit_tags(tab, table.buckets, table.shift, table.tag_shift, cand, cand >= 0, lossy)
                                    : visit(tab, table.buckets / 2, cand, cand >= 0, lossy);
             const unsigned m = __ballot_sync(0xffffffffu, fresh);
