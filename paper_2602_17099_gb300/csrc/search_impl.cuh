@@ -666,9 +666,13 @@ search_kernel(const SearchArgs a, const TableShape table, int prefetch) {
 // evaluations.)  A tag costs some ten instructions more a lookup than an id, so short
 // lists keep ids (50k Gaussian rows, R 16, ef 128: 2,048 ids 1.13 ms, tags 1.22, 1,536 ids
 // 1.16); so do graphs whose ids need more than 15 bits beside the set.
+//
+// The latency shape takes up to 8,192 ids for launches that one CTA per SM holds, else
+// 6,144, with which two fit: 1,216 queries, ef 256, took two waves of 152 CTAs with more (50k
+// Gaussian rows of 8 dimensions, R 24: 1.07 ms, now 0.44; 30k embedding-like rows 6.7, 3.5).
 template <int VAR>
-TableShape table_shape(int ef, int r_in, int64_t n) {
-    constexpr int kMost = VAR == kLatencyShape ? 8192 : VAR == 1 ? 2048 : 1536;
+TableShape table_shape(int ef, int r_in, int64_t n, int64_t nq) {
+    const int most = VAR != kLatencyShape ? (VAR == 1 ? 2048 : 1536) : nq > kLatencyQueries / 2 ? 6144 : 8192;
     const int all = std::max(ef * r_in + ef * r_in / 4, 1024);
     TableShape t = {};
     if (VAR != kLatencyShape && ef > 64 && all > 2560) {
@@ -683,14 +687,14 @@ TableShape table_shape(int ef, int r_in, int64_t n) {
             return t;
         }
     }
-    const int slots = std::min(all, ef > 64 ? std::max(kMost, 2048) : kMost);
+    const int slots = std::min(all, ef > 64 ? std::max(most, 2048) : most);
     t.buckets = (uint32_t)(slots + 63) / 64 * 16;
     return t;
 }
 
 template <int F4, int EFMAX, int MODE, int VAR, bool JOBS>
 cudaError_t launch_t(const SearchArgs &a, int prefetch, cudaStream_t st) {
-    const TableShape table = table_shape<VAR>(a.ef, a.r_in, a.n_base);
+    const TableShape table = table_shape<VAR>(a.ef, a.r_in, a.n_base, a.nq);
     const size_t smem = (size_t)kSearchWarps * warp_smem_bytes(table.buckets, EFMAX, MODE == kCodeFilter ? F4 : 0);
     auto kern = search_kernel<F4, EFMAX, MODE, VAR, JOBS>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -60,3 +60,28 @@ def test_searches_on_both_sides_of_the_tags_range(rn, n):
     np.testing.assert_array_equal(ids.cpu().numpy(), want[0])
     keep = want[0] >= 0
     np.testing.assert_array_equal(dd.cpu().numpy()[keep], want[1][keep])
+
+
+def test_the_largest_latency_launch_is_one_wave(rn):
+    # 1,216 queries are two CTAs of four on each of 152 SMs: with beams of 256 and their
+    # tables both have to fit an SM's shared memory.  In two waves the launch takes twice
+    # as long as half of its queries (measured 2.4 times), in one little longer.
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    x = torch.randn(50_000, 8, generator=g, device="cuda")
+    adj, entry = rn.build_segment(x, 24, 48)
+    q = torch.randn(1216, 8, generator=g, device="cuda")
+    seeds = torch.full((1216, 1), entry, dtype=torch.int32, device="cuda")
+
+    def median_ms(nq):
+        times = []
+        for _ in range(15):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            rn.search(x, adj, q[:nq], seeds[:nq], 256, 10)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b))
+        return sorted(times)[7]
+
+    assert median_ms(1216) < 1.7 * median_ms(608)
