@@ -110,3 +110,24 @@ def test_coded_merge_build_and_expand_equal_fp32(rn, monkeypatch, kind):
     for mode in (1, 2):
         for a, b in zip(out[mode], out[0]):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("d", [64, 96, 128, 256, 768])
+@pytest.mark.parametrize("kind,mode", [("bytes", 2), ("unit", 1), ("outlier", 0)])
+def test_the_searches_run_in_the_mode_that_the_rows_allow(rn, monkeypatch, d, kind, mode):
+    # the kernel's third template argument: 0 FP32 rows, 1 codes first, 2 codes alone (not
+    # at 768 dimensions, whose distances can exceed 2^24)
+    from torch.profiler import ProfilerActivity, profile
+    rng = np.random.default_rng(d)
+    X = _rows(kind, 2001, d, rng)
+    adj = _graph(len(X), 32, rng)
+    Q = X[rng.integers(8, len(X), NQ)].copy()
+    seeds = rng.integers(0, len(X), size=(NQ, 1)).astype(np.int32)
+    _search(rn, monkeypatch, 2, X, adj, Q, seeds, 64, 10, rn.L2)
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        _search(rn, monkeypatch, 2, X, adj, Q, seeds, 64, 10, rn.L2)
+        torch.cuda.synchronize()
+    names = [e.key for e in prof.key_averages() if "search_kernel<" in e.key]
+    want = 1 if d == 768 and mode == 2 else mode
+    for name in names:                         # (none where kernels cannot be traced)
+        assert name.split("search_kernel<")[1].split(",")[2].strip() == str(want), name
