@@ -28,9 +28,9 @@
 // The uncovered vertices are listed anew every round, and the last rounds, few
 // vertices each, run in one launch of one thread-block cluster, which needs no host
 // between rounds (all rounds of up to kTailMax vertices run there, of up to kSmallMax in
-// one block; with 6 rounds over the whole grid before it instead of 16, 500k rows left
-// it 1.5 ms of work).  What is left is the chain of dependent loads of each round, some
-// 11 us.  S3 of 5,000 Gaussian rows 2.14 -> 0.41 ms, 2 x 500k SIFT-like rows 1.55 -> 0.81 ms, 300k
+// one block; larger segments go on over the whole grid until that few are left, see
+// launch_select_pivots).  What is left is the chain of dependent loads of each round, some
+// 11 us.  S3 of 5,000 Gaussian rows 2.14 -> 0.41 ms, 2 x 500k SIFT-like rows 1.55 -> 0.71 ms, 300k
 // DEEP-like rows in 5 segments 3.25 -> 1.90 ms.
 
 #include <cooperative_groups.h>
@@ -44,7 +44,8 @@ namespace {
 constexpr int32_t kCovered = -(1 << 30);   // gain of a covered vertex (and below)
 constexpr int64_t kTailMax = 32768;
 constexpr int kWide = 24;                  // reverse lists from here on take a warp
-constexpr int kFullRounds = 16;            // rounds over the whole grid before the cluster's
+constexpr int kFullRounds = 16;            // rounds over the whole grid at a time
+constexpr int64_t kNoLook = 98304;         // see launch_select_pivots
 // 16 bytes of state each in one block's shared memory.  One block and the cluster, whole
 // calls: 6,144 and 6,145 DEEP-like rows 226 and 238 us, Gaussian ones (36 rounds) 494 and 544;
 // at 8,001 rows the cluster is ahead (318 against 348 us for S3 of a merge).
@@ -89,6 +90,28 @@ __device__ __forceinline__ void put(T *p, int32_t v) {
     else __stcg(p, v);
 }
 
+// The vote of the uncovered z, of gain gz.
+template <bool kShared>
+__device__ __forceinline__ void vote(const PivotState &s, int32_t z, int32_t gz) {
+    put<kShared>(s.snap + z, gz);
+    int32_t best = z, gb = gz;
+    int weight = 1;   // z's own
+    const int32_t *nz = s.nplus + (int64_t)z * s.k_plus;
+#pragma unroll 5
+    for (int j = 0; j < s.k; ++j) {
+        const int32_t y = __ldg(nz + j);
+        if (y < 0) continue;
+        const int32_t gy = get<kShared>(s.gain + y);
+        if (y == best) ++weight;
+        else if (gy > gb || (gy == gb && gy >= 0 && y < best)) {
+            best = y;
+            gb = gy;
+            weight = 1;
+        }
+    }
+    atomicAdd(s.votes + best, weight);
+}
+
 // Lists the uncovered vertices of cur[0..nc) in next and takes their votes;
 // thread t of `threads` (whole warps).
 template <bool kShared, class T>
@@ -106,23 +129,7 @@ __device__ __forceinline__ void vote_phase(const PivotState &s, const T *cur, in
         base = __shfl_sync(0xffffffffu, base, 0);
         if (!open) continue;
         put<kShared>(next + base + __popc(m & lanemask_lt()), z);
-        put<kShared>(s.snap + z, gz);
-        int32_t best = z, gb = gz;
-        int weight = 1;   // z's own
-        const int32_t *nz = s.nplus + (int64_t)z * s.k_plus;
-#pragma unroll 5
-        for (int j = 0; j < s.k; ++j) {
-            const int32_t y = __ldg(nz + j);
-            if (y < 0) continue;
-            const int32_t gy = get<kShared>(s.gain + y);
-            if (y == best) ++weight;
-            else if (gy > gb || (gy == gb && gy >= 0 && y < best)) {
-                best = y;
-                gb = gy;
-                weight = 1;
-            }
-        }
-        atomicAdd(s.votes + best, weight);
+        vote<kShared>(s, z, gz);
     }
 }
 
@@ -206,10 +213,35 @@ __device__ __forceinline__ void select_phase(const PivotState &s, const T *next,
     }
 }
 
+// The same over the whole grid.  A block appends its 256 entries at once: the list's order,
+// which decides how far the rounds' accesses lie apart, breaks up eight times later than
+// with an append a warp (4M DEEP-like rows 25.6 -> 15.2 ms, 500k SIFT-like ones 0.80 -> 0.70).
 __global__ void __launch_bounds__(256) piv_vote_kernel(PivotState s, const int32_t *cur, int32_t *next, PivotCtl *ctl,
                                                        int round) {
-    vote_phase<false>(s, cur, ctl->count[round], next, &ctl->count[round + 1], blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
-               (int64_t)gridDim.x * blockDim.x);
+    __shared__ int32_t count[8], base;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t nc = ctl->count[round];
+    for (int64_t i0 = blockIdx.x * (int64_t)256; i0 < nc; i0 += (int64_t)gridDim.x * 256) {
+        const int64_t i = i0 + threadIdx.x;
+        const int32_t z = i < nc ? get<false>(cur + i) : -1;
+        const int32_t gz = z >= 0 ? get<false>(s.gain + z) : kCovered;
+        const bool open = gz >= 0;
+        const unsigned m = __ballot_sync(0xffffffffu, open);
+        if (lane == 0) count[warp] = __popc(m);
+        __syncthreads();
+        int before = 0, all = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            before += w < warp ? count[w] : 0;
+            all += count[w];
+        }
+        if (threadIdx.x == 0) base = all ? atomicAdd(&ctl->count[round + 1], all) : 0;
+        __syncthreads();
+        if (open) {
+            put<false>(next + base + before + __popc(m & lanemask_lt()), z);
+            vote<false>(s, z, gz);
+        }
+    }
 }
 
 __global__ void __launch_bounds__(256) piv_select_kernel(PivotState s, const int32_t *next, PivotCtl *ctl, int round) {
@@ -369,18 +401,35 @@ cudaError_t launch_select_pivots(const int32_t *nplus, int64_t n, int32_t k_plus
     int32_t *cur = pivots, *next = followers;
     const int g = grid_n(n);
     piv_init_kernel<<<g, 256, 0, st>>>(s, n, cur, ctl);
+    // Rounds over the whole grid, sixteen at a time, until few enough are left for the
+    // cluster's eight SMs: looked at (a wait, some 15 us) for segments over kNoLook.  Sixteen
+    // rounds leave SIFT-like rows almost nothing at 500k, but most of 4M DEEP-like rows (52
+    // rounds: 99.9 ms with the rest in the cluster, 15.2 now) and of Gaussian ones (500k, 124
+    // rounds: 53.6 and 5.8 ms; 75k, not looked at: 3.6).
     int round = 0;
-    if (n > kTailMax)
-        for (; round < kFullRounds; ++round) {
+    int32_t left = (int32_t)n;
+    while (n > kTailMax) {
+        for (round = 0; round < kFullRounds; ++round) {
             piv_vote_kernel<<<g, 256, 0, st>>>(s, cur, next, ctl, round);
             piv_select_kernel<<<g, 256, 0, st>>>(s, next, ctl, round);
             int32_t *sw = cur;
             cur = next;
             next = sw;
         }
+        note_launches(2 * round);
+        if (n <= kNoLook) break;
+        const int32_t before = left;
+        cudaError_t e = cudaMemcpyAsync(&left, &ctl->count[round], sizeof(left), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return e;
+        if (left <= kTailMax || left >= before) break;   // (no progress: the cluster's kernel reports it)
+        e = cudaMemcpyAsync(&ctl->count[0], &ctl->count[round], sizeof(left), cudaMemcpyDeviceToDevice, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(&ctl->count[1], 0, sizeof(ctl->count) - sizeof(left), st);
+        if (e != cudaSuccess) return e;
+    }
     piv_tail_kernel<<<kTailBlocks, kTailThreads, 0, st>>>(s, cur, next, ctl, round);
     piv_compact_kernel<<<g, 256, 0, st>>>(n, pivot_of, pivots, followers, ctl);
-    note_launches(3 + 2 * round);
+    note_launches(3);
     return cudaGetLastError();
 }
 
